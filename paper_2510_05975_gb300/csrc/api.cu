@@ -280,6 +280,10 @@ struct KnnInputs {
   // locality order of the tensor-core operands (tc_rows / tc_cols / nb_cols hold positions)
   const int32_t* perm;
   int wave_start;
+  ResShape res;                           // res.kt > 0: tc_rows / tc_cols are tile images,
+  const int32_t* col_perm = nullptr;      // columns in a sampled order (col_pos: its inverse)
+  const int32_t* col_pos = nullptr;
+  int64_t part_count[RES_PARTS] = {0, 0, 0, 0};
   int variant = -1;  // tensor-core screen pipeline variant (-1: autotuned)
   const uint8_t* u8 = nullptr;  // 8-bit rows of the points (rows = columns), or null
   int u8w = 0;
@@ -314,6 +318,10 @@ static cng_status run_knn(const KnnInputs& in, int32_t* out_ids, float* out_dist
     ta.perm = in.perm;
     ta.wave_start = in.wave_start;
     ta.variant = in.variant;
+    ta.res = in.res;
+    ta.col_perm = in.col_perm;
+    ta.col_pos = in.col_pos;
+    for (int i = 0; i < RES_PARTS; ++i) ta.part_count[i] = in.part_count[i];
     CK(pool.alloc(&ta.rowbuf, ta.rowbuf_words));
     std::string msg;
     if (in.variant < 0) {  // a first use of this shape times the variants (outside the timing)
@@ -328,7 +336,8 @@ static cng_status run_knn(const KnnInputs& in, int32_t* out_ids, float* out_dist
     sm.rb = in.rb_rows;
     sm.rbmax = in.rbmax;
     sm.normmax = in.normmax;
-    sm.acc_err = (float)(in.kpad + 8) * 1.1920929e-7f;  // K terms, 2^-23 per add
+    // K terms, 2^-23 per add (the norm pieces among them when they are part of the operands)
+    sm.acc_err = (float)(in.res.kt > 0 ? in.res.kt + 16 : in.kpad + 8) * 1.1920929e-7f;
     sm.scale2 = in.scale2;
   } else {
     int cpl = 0;
@@ -441,11 +450,84 @@ static cng_status prepare(DevPool& pool, const void* pts_dev, int dtype, int64_t
   return CNG_OK;
 }
 
-// Self k-NN through the tensor-core screen in a locality order: replaces pr's screening copy by
-// one in k-d order and points ki at it (rows and columns are positions, ki->perm the ids).
+static float key_to_float(uint32_t k) {
+  uint32_t b = (k & 0x80000000u) ? (k & 0x7fffffffu) : ~k;
+  float f;
+  memcpy(&f, &b, 4);
+  return f;
+}
+static float bits_to_float(uint32_t b) {
+  float f;
+  memcpy(&f, &b, 4);
+  return f;
+}
+
+// The columns' tile image in a sampled order of perm (device ids; *order: position -> id, *pos: its
+// inverse if wanted) and the parts' sizes, for screens whose rows fit the resident kernel.
+// Synchronises.
+static cng_status sampled_image(DevPool& pool, const ResShape& r, int fp16, const Prepared& pr,
+                                int64_t n, int kpad, const int32_t* perm, void** image,
+                                const int32_t** order, const int32_t** pos, int64_t* part_count,
+                                cudaStream_t s) {
+  int32_t *out, *inv = nullptr, *cnt;
+  char *scr, *img;
+  CK(pool.alloc(&out, (size_t)n));
+  if (pos) CK(pool.alloc(&inv, (size_t)n));
+  CK(pool.alloc(&cnt, 4));
+  CK(pool.alloc(&scr, sample_scratch_bytes(n)));
+  CK(launch_sample_order(perm, n, out, inv, cnt, scr, s));
+  CK(pool.alloc(&img, res_image_bytes(r, n)));
+  CK(launch_tile_image(r, fp16 != 0, pr.tc, kpad, pr.nb, out, n, img, s));
+  int32_t h[4];
+  CK(cudaMemcpyAsync(h, cnt, sizeof(h), cudaMemcpyDeviceToHost, s));
+  CK(cudaStreamSynchronize(s));
+  for (int i = 0; i < RES_PARTS; ++i) part_count[i] = h[i];
+  *image = img;
+  *order = out;
+  if (pos) *pos = inv;
+  return CNG_OK;
+}
+
+// Self k-NN through the tensor-core screen: replaces pr's screening copy by one in sweep order and
+// points ki at it.  kd: a k-d locality order (*ms its time).  Rows that fit the resident kernel
+// have two copies: the rows in k-d (or input) order, so that the rows of a block share most of
+// their near columns, and the columns in a sampled order on top of it.
 static cng_status apply_order(DevPool& pool, Prepared* pr, int dtype, int64_t n, int d, int dpad,
-                              int kpad, KnnInputs* ki, double* ms, cudaStream_t s) {
-  if (order_levels(n) == 0) return CNG_OK;
+                              int kpad, int kd, KnnInputs* ki, double* ms, cudaStream_t s) {
+  kd = kd && order_levels(n) > 0;
+  ResShape res;
+  if (res_shape(d, bits_to_float(pr->st.nbmax_bits), &res)) {
+    Timer to(s);
+    to.mark();
+    int32_t* perm;
+    void* cimg;
+    char* rimg;
+    CK(pool.alloc(&perm, (size_t)n));
+    if (kd) {
+      char* oscr;
+      CK(pool.alloc(&oscr, order_scratch_bytes(n)));
+      CK(launch_order(pr->xs, dtype, n, d, dpad, perm, oscr, s));
+    } else {
+      CK(launch_iota(perm, n, s));
+    }
+    CK(pool.alloc(&rimg, res_image_bytes(res, n)));
+    CK(launch_tile_image(res, ki->tc_fp16 != 0, pr->tc, kpad, pr->nb, perm, n, rimg, s));
+    cng_status st = sampled_image(pool, res, ki->tc_fp16, *pr, n, kpad, perm, &cimg, &ki->col_perm,
+                                  &ki->col_pos, ki->part_count, s);
+    if (st != CNG_OK) return st;
+    to.mark();
+    CK(cudaStreamSynchronize(s));
+    cudaFree(pr->tc);
+    pool.release(pr->tc);
+    pr->tc = rimg;
+    ki->tc_rows = rimg;
+    ki->tc_cols = cimg;
+    ki->res = res;
+    ki->perm = perm;
+    if (kd) *ms = to.ms(0, 1);
+    return CNG_OK;
+  }
+  if (!kd) return CNG_OK;
   Timer to(s);
   to.mark();
   int32_t* perm;
@@ -473,18 +555,6 @@ static cng_status apply_order(DevPool& pool, Prepared* pr, int dtype, int64_t n,
   ki->wave_start = 1;
   *ms = to.ms(0, 1);
   return CNG_OK;
-}
-
-static float key_to_float(uint32_t k) {
-  uint32_t b = (k & 0x80000000u) ? (k & 0x7fffffffu) : ~k;
-  float f;
-  memcpy(&f, &b, 4);
-  return f;
-}
-static float bits_to_float(uint32_t b) {
-  float f;
-  memcpy(&f, &b, 4);
-  return f;
 }
 
 // 8-bit rows u = x - min(x) hold the data exactly when every coordinate is an integer and the
@@ -677,8 +747,8 @@ extern "C" cng_status cng_build(const void* points, int32_t dtype, int64_t n, in
   TcShape tshape{-1, -1, -1, -1};
   // locality order of the screen's operands (speed only; the lists are exact either way)
   double ms_order = 0;
-  if (screen == CNG_SCREEN_TC && !P.input_order) {
-    st = apply_order(pool, &pr, dtype, n, d, dpad, kpad, &ki, &ms_order, s);
+  if (screen == CNG_SCREEN_TC) {
+    st = apply_order(pool, &pr, dtype, n, d, dpad, kpad, !P.input_order, &ki, &ms_order, s);
     if (st != CNG_OK) return st;
   }
   // integer data spanning <= 255: 8-bit rows for exact integer pair distances in the rerank
@@ -1576,8 +1646,22 @@ extern "C" cng_status cng_knn(const float* base, int64_t n, const float* rows, i
   ki.normmax = std::sqrt(bits_to_float(both.nbmax_bits));
   double ms_order = 0;
   if (self && screen == CNG_SCREEN_TC) {
-    st = apply_order(pool, &pb, CNG_F32, n, d, dpad, kpad, &ki, &ms_order, s);
+    st = apply_order(pool, &pb, CNG_F32, n, d, dpad, kpad, 1, &ki, &ms_order, s);
     if (st != CNG_OK) return st;
+  } else if (screen == CNG_SCREEN_TC &&
+             res_shape(d, bits_to_float(pb.st.nbmax_bits), &ki.res)) {
+    void* cimg;
+    char* rimg;
+    int32_t* input;
+    CK(pool.alloc(&input, (size_t)n));
+    CK(launch_iota(input, n, s));
+    st = sampled_image(pool, ki.res, ki.tc_fp16, pb, n, kpad, input, &cimg, &ki.col_perm, nullptr,
+                       ki.part_count, s);
+    if (st != CNG_OK) return st;
+    CK(pool.alloc(&rimg, res_image_bytes(ki.res, m)));
+    CK(launch_tile_image(ki.res, ki.tc_fp16 != 0, prw.tc, kpad, prw.nb, nullptr, m, rimg, s));
+    ki.tc_rows = rimg;
+    ki.tc_cols = cimg;
   }
   double ms_screen = 0, ms_rerank = 0;
   st = run_knn(ki, ids, dists, ctr, &ms_screen, &ms_rerank, s);
@@ -1632,6 +1716,15 @@ static cng_status tc_scores(const float* rows, int64_t m, const float* cols, int
   ta.status = status;
   ta.rowbuf_words = screen_tc_rowbuf_words(m, n, 32);
   CK(pool.alloc(&ta.rowbuf, ta.rowbuf_words));
+  if (res_shape(d, bits_to_float(pc.st.nbmax_bits), &ta.res)) {
+    char *ri, *ci;
+    CK(pool.alloc(&ri, res_image_bytes(ta.res, m)));
+    CK(pool.alloc(&ci, res_image_bytes(ta.res, n)));
+    CK(launch_tile_image(ta.res, fp16 != 0, pr.tc, kpad, pr.nb, nullptr, m, ri, s));
+    CK(launch_tile_image(ta.res, fp16 != 0, pc.tc, kpad, pc.nb, nullptr, n, ci, s));
+    ta.A = ri;
+    ta.B = ci;
+  }
   std::string msg;
   cudaError_t e = launch_screen_tc_dump(ta, scores, s, &msg);
   if (e != cudaSuccess) return fail(CNG_E_CUDA, "tensor-core screen: " + msg + cudaGetErrorString(e));

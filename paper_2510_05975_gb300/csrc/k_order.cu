@@ -353,6 +353,67 @@ cudaError_t launch_order(const void* xs, int dtype, int64_t n, int d, int dpad, 
   return cudaGetLastError();
 }
 
+// ---- sampled order ------------------------------------------------------------------------------
+// part of an id: 0 for 1 in 64 ids, 1 up to 1 in 16, 2 up to 1 in 4, else 3, from a hash of the id
+// alone, so that whatever structure the data has, each part is a random sample of any point's
+// neighbours.
+__global__ void __launch_bounds__(256) smp_key_kernel(const int32_t* __restrict__ perm, int64_t n,
+                                                      uint32_t* __restrict__ key, int32_t* counts) {
+  __shared__ int c[4];
+  if (threadIdx.x < 4) c[threadIdx.x] = 0;
+  __syncthreads();
+  int mine[4] = {0, 0, 0, 0};
+  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n;
+       p += (int64_t)gridDim.x * blockDim.x) {
+    const uint32_t u = ord_mix((uint32_t)perm[p] * 0x9e3779b9u + 0x3c6ef372u) & 63u;
+    const int k = u == 0u ? 0 : (u < 4u ? 1 : (u < 16u ? 2 : 3));
+    key[p] = (uint32_t)k;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) mine[i] += k == i;
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    if (mine[i]) atomicAdd(&c[i], mine[i]);
+  __syncthreads();
+  if (threadIdx.x < 4 && c[threadIdx.x]) atomicAdd(&counts[threadIdx.x], c[threadIdx.x]);
+}
+
+size_t sample_scratch_bytes(int64_t n) {
+  const int64_t nblk = (n + RS_TILE - 1) / RS_TILE;
+  return 2 * (((size_t)n * 4 + 255) & ~size_t(255)) + (size_t)256 * nblk * 4;
+}
+
+__global__ void smp_invert_kernel(const int32_t* __restrict__ order, int64_t n, int32_t* __restrict__ pos) {
+  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n;
+       p += (int64_t)gridDim.x * blockDim.x)
+    pos[order[p]] = (int32_t)p;
+}
+
+cudaError_t launch_sample_order(const int32_t* perm, int64_t n, int32_t* out, int32_t* pos,
+                                int32_t* counts_dev, void* scratch, cudaStream_t s) {
+  const int nblk = (int)((n + RS_TILE - 1) / RS_TILE);
+  const size_t kb = ((size_t)n * 4 + 255) & ~size_t(255);
+  uint32_t* key = static_cast<uint32_t*>(scratch);
+  uint32_t* key2 = reinterpret_cast<uint32_t*>(static_cast<char*>(scratch) + kb);
+  uint32_t* ghist = reinterpret_cast<uint32_t*>(static_cast<char*>(scratch) + 2 * kb);
+  cudaError_t e = cudaMemsetAsync(counts_dev, 0, 4 * sizeof(int32_t), s);
+  if (e != cudaSuccess) return e;
+  const int grid = (int)std::min<int64_t>((n + 255) / 256, (int64_t)num_sms() * 8);
+  count_launch();
+  smp_key_kernel<<<grid, 256, 0, s>>>(perm, n, key, counts_dev);
+  count_launch();
+  rs_hist_kernel<<<nblk, RS_THREADS, 0, s>>>(key, n, 0, nblk, ghist);
+  count_launch();
+  rs_scan_kernel<<<1, 1024, 0, s>>>(ghist, (int64_t)4 * nblk);  // digits 0..3 alone
+  count_launch();
+  rs_scatter_kernel<<<nblk, RS_THREADS, 0, s>>>(key, perm, key2, out, n, 0, nblk, ghist);
+  if (pos) {
+    count_launch();
+    smp_invert_kernel<<<grid, 256, 0, s>>>(out, n, pos);
+  }
+  return cudaGetLastError();
+}
+
 cudaError_t launch_order_gather(const void* xi, const float* nbi, const int32_t* perm, int64_t n,
                                 int kpad, void* xo, float* nbo, cudaStream_t s) {
   const int row_vecs = kpad * 2 / 16;

@@ -1,16 +1,15 @@
-// k_screen_tc.cu -- tensor-core candidate screen (K1) for sm_103a: tcgen05.mma with TMEM
-// accumulators, TMA tile loads into 128-byte-swizzled shared memory, mbarrier pipelines and
-// a fused per-row top-L' filter.  It yields, for each row point x, a superset list of its
-// nearest columns y by the screened score  s(x,y) = ||y_b||^2 - 2 <x_b, y_b>,  which differs
-// from ||x_b - y_b||^2 only by the row constant ||x_b||^2 (x_b, y_b: bf16-rounded operands;
-// fp16 operands for fp16 data).  The rerank (K2) recomputes FP32 distances and certifies
+// k_screen_tc.cu -- tensor-core candidate screen (K1) for rows wider than the resident kernel
+// takes (k_screen_res.cu: up to 250 coordinates; also rows whose norms its operands cannot hold):
+// tcgen05.mma with TMEM accumulators, TMA tile loads into 128-byte-swizzled shared memory, mbarrier
+// pipelines and a fused per-row top-L' filter.  It yields, for each row point x, a superset list
+// of its nearest columns y by the screened score  s(x,y) = ||y_b||^2 - 2 <x_b, y_b>,  which
+// differs from ||x_b - y_b||^2 only by the row constant ||x_b||^2 (x_b, y_b: bf16-rounded
+// operands; fp16 operands for fp16 data).  The rerank (K2) recomputes FP32 distances and certifies
 // the list; rows it cannot certify are rescanned exactly.
 //
 // CTA organisation (one CTA per SM, persistent over 256-row blocks):
-//   warp 8      TMA producer: for kpad <= 192 the row block's A tile once, then B tiles of 128
-//               columns with their column norms through an NST-stage ring (full / empty
-//               mbarriers); for wider rows A and B together in 64-wide K chunks through the
-//               same ring, and each tile's 128 column norms into a 4-slot norm ring
+//   warp 8      TMA producer: A and B together in 64-wide K chunks through an NST-stage ring (full /
+//               empty mbarriers), and each tile's 128 column norms into a 4-slot norm ring
 //   warp 9      TMEM owner (512 columns) and MMA issuer: per B tile, two M=128 x N=128
 //               accumulators (rows 0-127 and 128-255), K in steps of 16, into one of two TMEM
 //               buffers; tcgen05.commit frees each operand stage and publishes the buffer
@@ -28,6 +27,7 @@
 #include "launch_count.h"
 #include "cng_internal.h"
 #include "device_common.cuh"
+#include "screen_common.cuh"
 #include "screen_tc.h"
 
 #include <mutex>
@@ -41,18 +41,14 @@ constexpr int TC_NBUF = 512 / (2 * TC_BN);  // accumulator buffers in the 512 TM
 constexpr int TC_NBUF_LOG = TC_NBUF == 4 ? 2 : 1;
 constexpr int TC_MAXST = TC_BN == 64 ? 8 : 4;  // operand stages at most
 constexpr int TC_NR = 4;            // column-norm ring slots (tiles whose norms are in flight)
-static_assert((2 * TC_MAXST + 2 * TC_NBUF + 2 * TC_NR + 3) * 8 + 8 <= 256,
+static_assert((2 * TC_MAXST + 2 * TC_NBUF + 2 * TC_NR + 1) * 8 + 8 <= 256,
               "barrier block exceeds its 256 bytes");
-static_assert(TC_MAXST >= TC_NR, "the column-norm area holds max(stages, ring slots) tiles");
 static_assert(TC_NBUF == 2 || TC_NBUF == 4, "two or four accumulator buffers");
 constexpr int TC_KC = 64;           // K elements per 128-byte swizzle chunk
 constexpr int TC_SLACK = 16;        // keys past the Lp-th a thinning may keep (one digit pass)
 constexpr int TC_THREADS = 320;     // 8 epilogue warps + producer + MMA
 constexpr int TC_PRODUCER = 8;
 constexpr int TC_MMA = 9;
-// wait iterations before declaring a timeout (each try_wait may suspend the thread for a
-// system-dependent time; no suspend-time hint, so a completed phase is seen at once)
-constexpr uint32_t TC_SPIN = 1u << 19;
 
 struct TcParams {
   int64_t m, n;
@@ -72,35 +68,7 @@ struct TcParams {
   int sync_d;           // checkpoint lag in windows
 };
 
-// Producers meet at checkpoints every TC_SYNC_K tiles of their own sequence; a producer at
-// checkpoint c waits until every CTA that reaches checkpoint c - sync_d has reached it, so
-// the CTAs of a wave stay within sync_d * TC_SYNC_K B tiles of each other and share the tiles
-// through L2 instead of each streaming them from DRAM.  The wait only serves the cache: it is
-// bounded (about 2 ms) and the producer proceeds when it expires.
-constexpr int TC_SYNC_K = 256 * 128 / TC_BN;  // tiles per checkpoint window (32,768 columns)
-constexpr uint32_t TC_SYNC_SPIN = 8192;
-
-CNG_DEV uint32_t ld_acquire_u32(const uint32_t* p) {
-  uint32_t v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-
-CNG_DEV void wave_checkpoint(const TcParams& P, int64_t it, int64_t nrb, int ntiles) {
-  if (!P.sync || it == 0 || it % TC_SYNC_K != 0) return;
-  const int64_t c = it / TC_SYNC_K;
-  atomicAdd(&P.sync[c], 1u);
-  if (c <= P.sync_d) return;
-  const int64_t cw = c - P.sync_d;
-  // CTAs reaching tile index cw * K: those with a row block in wave (cw * K) / ntiles
-  const int64_t w = (cw * TC_SYNC_K) / ntiles;
-  const int64_t left = nrb - w * (int64_t)gridDim.x;
-  const uint32_t expect = (uint32_t)(left < 0 ? 0 : (left > gridDim.x ? gridDim.x : left));
-  for (uint32_t i = 0; i < TC_SYNC_SPIN; ++i) {
-    if (ld_acquire_u32(&P.sync[cw]) >= expect) return;
-    __nanosleep(200);
-  }
-}
+constexpr int TC_SYNC_K = TC_SYNC_COLS / TC_BN;  // tiles per checkpoint window
 
 // First column tile of row block rb's sweep.  A wave is the gridDim.x consecutive row blocks
 // processed together; all its CTAs share the start, so B tiles stay shared through L2.
@@ -111,68 +79,12 @@ CNG_DEV int sweep_start(const TcParams& P, int64_t rb, int ntiles) {
   return t0 < ntiles ? (int)t0 : ntiles - 1;
 }
 
-// ---- PTX wrappers ------------------------------------------------------------------------------
-CNG_DEV uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-CNG_DEV void mbar_init(uint64_t* b, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count) : "memory");
-}
-CNG_DEV void mbar_expect_tx(uint64_t* b, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(b)), "r"(bytes)
-               : "memory");
-}
-CNG_DEV void mbar_arrive(uint64_t* b) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(b)) : "memory");
-}
-CNG_DEV bool mbar_try(uint64_t* b, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok)
-      : "r"(smem_u32(b)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// Bounded wait; returns false (and raises the CTA abort flag) on expiry or if aborted.
-CNG_DEV bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* abort_flag, uint32_t* status) {
-  for (uint32_t i = 0; i < TC_SPIN; ++i) {
-    if (mbar_try(b, parity)) return true;
-    if ((i & 15u) == 15u && *abort_flag) return false;
-  }
-  *abort_flag = 1;
-  atomicOr(status, ST_TIMEOUT);
-  return false;
-}
-
-// Warp-uniform bounded wait: every lane polls, the warp proceeds only when all lanes saw the
-// phase complete, so the whole warp leaves together (needed before .sync.aligned TMEM loads).
-CNG_DEV bool mbar_wait_warp(uint64_t* b, uint32_t parity, volatile int* abort_flag, uint32_t* status,
-                            uint32_t spin = TC_SPIN) {
-  for (uint32_t i = 0; i < spin; ++i) {
-    if (__all_sync(FULL, mbar_try(b, parity))) return true;
-    if ((i & 15u) == 15u && __any_sync(FULL, *abort_flag != 0)) return false;
-  }
-  if ((threadIdx.x & 31) == 0) {
-    *abort_flag = 1;
-    atomicOr(status, ST_TIMEOUT);
-  }
-  __syncwarp();
-  return false;
-}
-
+// ---- PTX wrappers (the others are in screen_common.cuh) -----------------------------------------
 CNG_DEV void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
           smem_u32(dst)),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar))
-      : "memory");
-}
-
-CNG_DEV void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-          smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(smem_u32(bar))
       : "memory");
 }
 
@@ -194,14 +106,6 @@ CNG_DEV void mma_f16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, ui
       "l"(a), "l"(b), "r"(idesc), "r"(acc)
       : "memory");
 }
-CNG_DEV void mma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                   smem_u32(bar))
-               : "memory");
-}
-CNG_DEV void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-CNG_DEV void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
 CNG_DEV void tmem_ld32(uint32_t taddr, float* v) {
   uint32_t r[32];
   asm volatile(
@@ -513,12 +417,9 @@ CNG_DEV void process_chunk(uint32_t* r, int64_t cb, bool edge, bool live, int64_
 }
 
 // ---- the kernel --------------------------------------------------------------------------------
-// KSTREAM = false: the row block's A tile stays resident (kpad <= 192) and each stage holds one
-//   B tile of TC_BN columns x kpad.
-// KSTREAM = true: A and B are streamed together in 64-wide K chunks (any kpad), each stage
-//   holding the row block's A chunk and the column tile's B chunk; the accumulators sum the
-//   chunks of a tile in TMEM.
-template <int CPL, bool DUMP, bool KSTREAM>
+// A and B are streamed together in 64-wide K chunks (any kpad), each stage holding the row block's
+// A chunk and the column tile's B chunk; the accumulators sum the chunks of a tile in TMEM.
+template <int CPL, bool DUMP>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 screen_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                  TcParams P, float* dump) {
@@ -526,22 +427,17 @@ screen_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
   // 1024-byte aligned tile region
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const int a_bytes = KSTREAM ? 0 : TC_BM * P.kpad * 2;
-  const int stage_bytes = KSTREAM ? (TC_BM + TC_BN) * TC_KC * 2 : TC_BN * P.kpad * 2;
-  unsigned char* sA = smem;
-  unsigned char* sB = smem + a_bytes;
-  // column norms: per operand stage with a resident A tile, else a TC_NR-slot ring
-  float* sNB = reinterpret_cast<float*>(sB + P.nst * stage_bytes);  // [max(nst, TC_NR)][TC_BN]
-  uint64_t* bars = reinterpret_cast<uint64_t*>(sNB + TC_MAXST * TC_BN);
+  const int stage_bytes = (TC_BM + TC_BN) * TC_KC * 2;
+  unsigned char* sB = smem;
+  float* sNB = reinterpret_cast<float*>(sB + P.nst * stage_bytes);  // column norms [TC_NR][TC_BN]
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sNB + TC_NR * TC_BN);
   uint64_t* b_full = bars;               // [nst]
   uint64_t* b_empty = bars + P.nst;      // [nst]
   uint64_t* t_full = bars + 2 * P.nst;   // [TC_NBUF]
   uint64_t* t_empty = t_full + TC_NBUF;  // [TC_NBUF]
   uint64_t* n_full = t_empty + TC_NBUF;  // [TC_NR]
   uint64_t* n_empty = n_full + TC_NR;    // [TC_NR]
-  uint64_t* a_full = n_empty + TC_NR;    // [1]
-  uint64_t* a_empty = a_full + 1;        // [1]
-  uint64_t* fin = a_empty + 1;           // [1] MMA drain at exit
+  uint64_t* fin = n_empty + TC_NR;       // [1] MMA drain at exit
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(fin + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   uint32_t* hist_all = reinterpret_cast<uint32_t*>(reinterpret_cast<unsigned char*>(bars) + 256);  // [8][256]
@@ -553,9 +449,7 @@ screen_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
   if (tid == 0) {
     for (int i = 0; i < P.nst; ++i) {
       mbar_init(&b_full[i], 1);
-      // the MMA's commit; with a resident A tile each stage also carries its tile's column
-      // norms, which the 8 epilogue warps release
-      mbar_init(&b_empty[i], KSTREAM ? 1 : 1 + 8);
+      mbar_init(&b_empty[i], 1);
     }
     for (int i = 0; i < TC_NBUF; ++i) {
       mbar_init(&t_full[i], 1);
@@ -565,8 +459,6 @@ screen_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
       mbar_init(&n_full[i], 1);
       mbar_init(&n_empty[i], 8);
     }
-    mbar_init(a_full, 1);
-    mbar_init(a_empty, 1);
     mbar_init(fin, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -587,61 +479,38 @@ screen_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&mapA)) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&mapB)) : "memory");
       int64_t it = 0;
-      int j = 0;
       int s = 0;         // stage of the next copy (advanced without dividing)
       uint32_t ph = 0;   // its phase
       int ns = 0;        // norm ring slot of the next tile
       uint32_t nph = 0;  // its phase
       bool ok = true;
-      for (int64_t rb = blockIdx.x; rb < nrb && ok; rb += gridDim.x, ++j) {
-        if (!KSTREAM) {
-          ok = mbar_wait(a_empty, (j & 1) ^ 1, abort_flag, P.status);
-          if (!ok) break;
-          mbar_expect_tx(a_full, (uint32_t)a_bytes);
-          for (int kc = 0; kc < P.nkc; ++kc)
-            tma_load_2d(sA + kc * (TC_BM * 128), &mapA, kc * TC_KC, (int)(rb * TC_BM), a_full);
-        }
+      for (int64_t rb = blockIdx.x; rb < nrb && ok; rb += gridDim.x) {
         const int t0 = sweep_start(P, rb, ntiles);
         for (int ti = 0; ti < ntiles; ++ti, ++it) {
           const int t = ti + t0 < ntiles ? ti + t0 : ti + t0 - ntiles;
-          wave_checkpoint(P, it, nrb, ntiles);
-          if (!KSTREAM) {
-            // the B tile and its column norms into one stage
+          wave_checkpoint(P.sync, P.sync_d, TC_SYNC_K, it, nrb, ntiles);
+          // the tile's column norms into the norm ring, then A and B in K chunks
+          ok = mbar_wait(&n_empty[ns], nph ^ 1, abort_flag, P.status);
+          if (!ok) break;
+          mbar_expect_tx(&n_full[ns], TC_BN * 4);
+          bulk_load(sNB + ns * TC_BN, P.nb + (int64_t)t * TC_BN, TC_BN * 4, &n_full[ns]);
+          if (++ns == TC_NR) {
+            ns = 0;
+            nph ^= 1u;
+          }
+          for (int kc = 0; kc < P.nkc && ok; ++kc) {
             ok = mbar_wait(&b_empty[s], ph ^ 1, abort_flag, P.status);
             if (!ok) break;
-            mbar_expect_tx(&b_full[s], (uint32_t)(stage_bytes + TC_BN * 4));
+            mbar_expect_tx(&b_full[s], (uint32_t)stage_bytes);
             unsigned char* dst = sB + s * stage_bytes;
-            for (int kc = 0; kc < P.nkc; ++kc)
-              tma_load_2d(dst + kc * (TC_BN * 128), &mapB, kc * TC_KC, t * TC_BN, &b_full[s]);
-            bulk_load(sNB + s * TC_BN, P.nb + (int64_t)t * TC_BN, TC_BN * 4, &b_full[s]);
+            tma_load_2d(dst, &mapA, kc * TC_KC, (int)(rb * TC_BM), &b_full[s]);
+            tma_load_2d(dst + TC_BM * 128, &mapB, kc * TC_KC, t * TC_BN, &b_full[s]);
             if (++s == P.nst) {
               s = 0;
               ph ^= 1u;
             }
-          } else {
-            // the tile's column norms into the norm ring, then A and B in K chunks
-            ok = mbar_wait(&n_empty[ns], nph ^ 1, abort_flag, P.status);
-            if (!ok) break;
-            mbar_expect_tx(&n_full[ns], TC_BN * 4);
-            bulk_load(sNB + ns * TC_BN, P.nb + (int64_t)t * TC_BN, TC_BN * 4, &n_full[ns]);
-            if (++ns == TC_NR) {
-              ns = 0;
-              nph ^= 1u;
-            }
-            for (int kc = 0; kc < P.nkc && ok; ++kc) {
-              ok = mbar_wait(&b_empty[s], ph ^ 1, abort_flag, P.status);
-              if (!ok) break;
-              mbar_expect_tx(&b_full[s], (uint32_t)stage_bytes);
-              unsigned char* dst = sB + s * stage_bytes;
-              tma_load_2d(dst, &mapA, kc * TC_KC, (int)(rb * TC_BM), &b_full[s]);
-              tma_load_2d(dst + TC_BM * 128, &mapB, kc * TC_KC, t * TC_BN, &b_full[s]);
-              if (++s == P.nst) {
-                s = 0;
-                ph ^= 1u;
-              }
-            }
-            if (!ok) break;
           }
+          if (!ok) break;
         }
       }
       if (!ok) {
@@ -659,36 +528,27 @@ screen_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
   } else if (warp == TC_MMA) {
     if (lane == 0) {
       int64_t tt = 0;
-      int j = 0;
       int s = 0;         // stage (advanced without dividing)
       uint32_t sph = 0;  // its phase
       bool ok = true;
-      for (int64_t rb = blockIdx.x; rb < nrb && ok; rb += gridDim.x, ++j) {
-        if (!KSTREAM) {
-          ok = mbar_wait(a_full, j & 1, abort_flag, P.status);
-          if (!ok) break;
-          tc_fence_after();
-        }
-        const uint32_t a_base = smem_u32(sA);
+      for (int64_t rb = blockIdx.x; rb < nrb && ok; rb += gridDim.x) {
         for (int t = 0; t < ntiles; ++t, ++tt) {
           const int b = (int)(tt & (TC_NBUF - 1));
           const uint32_t d_base = tmem + (uint32_t)(b * (2 * TC_BN));
-          if (!KSTREAM) {
+          ok = mbar_wait(&t_empty[b], (uint32_t)(((tt >> TC_NBUF_LOG) & 1) ^ 1), abort_flag, P.status);
+          if (!ok) break;
+          for (int kc = 0; kc < P.nkc && ok; ++kc) {
             ok = mbar_wait(&b_full[s], sph, abort_flag, P.status);
             if (!ok) break;
-            ok = mbar_wait(&t_empty[b], (uint32_t)(((tt >> TC_NBUF_LOG) & 1) ^ 1), abort_flag, P.status);
-            if (!ok) break;
             tc_fence_after();
-            const uint32_t b_base = smem_u32(sB + s * stage_bytes);
-            for (int kc = 0; kc < P.nkc; ++kc) {
+            const uint32_t st_base = smem_u32(sB + s * stage_bytes);
 #pragma unroll
-              for (int k16 = 0; k16 < TC_KC / 16; ++k16) {
-                const uint64_t bd = desc_sw128(b_base + kc * (TC_BN * 128) + k16 * 32);
+            for (int k16 = 0; k16 < TC_KC / 16; ++k16) {
+              const uint64_t bd = desc_sw128(st_base + TC_BM * 128 + k16 * 32);
 #pragma unroll
-                for (int acc = 0; acc < 2; ++acc) {
-                  const uint64_t ad = desc_sw128(a_base + kc * (TC_BM * 128) + acc * (128 * 128) + k16 * 32);
-                  mma_f16(d_base + (uint32_t)(acc * TC_BN), ad, bd, P.idesc, (kc | k16) != 0);
-                }
+              for (int acc = 0; acc < 2; ++acc) {
+                const uint64_t ad = desc_sw128(st_base + acc * (128 * 128) + k16 * 32);
+                mma_f16(d_base + (uint32_t)(acc * TC_BN), ad, bd, P.idesc, (kc | k16) != 0);
               }
             }
             mma_commit(&b_empty[s]);
@@ -696,35 +556,11 @@ screen_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
               s = 0;
               sph ^= 1u;
             }
-          } else {
-            ok = mbar_wait(&t_empty[b], (uint32_t)(((tt >> TC_NBUF_LOG) & 1) ^ 1), abort_flag, P.status);
-            if (!ok) break;
-            for (int kc = 0; kc < P.nkc && ok; ++kc) {
-              ok = mbar_wait(&b_full[s], sph, abort_flag, P.status);
-              if (!ok) break;
-              tc_fence_after();
-              const uint32_t st_base = smem_u32(sB + s * stage_bytes);
-#pragma unroll
-              for (int k16 = 0; k16 < TC_KC / 16; ++k16) {
-                const uint64_t bd = desc_sw128(st_base + TC_BM * 128 + k16 * 32);
-#pragma unroll
-                for (int acc = 0; acc < 2; ++acc) {
-                  const uint64_t ad = desc_sw128(st_base + acc * (128 * 128) + k16 * 32);
-                  mma_f16(d_base + (uint32_t)(acc * TC_BN), ad, bd, P.idesc, (kc | k16) != 0);
-                }
-              }
-              mma_commit(&b_empty[s]);
-              if (++s == P.nst) {
-                s = 0;
-                sph ^= 1u;
-              }
-            }
-            if (!ok) break;
           }
+          if (!ok) break;
           mma_commit(&t_full[b]);
         }
         if (!ok) break;
-        if (!KSTREAM) mma_commit(a_empty);
       }
       // drain every MMA this thread issued before TMEM is released
       mma_commit(fin);
@@ -738,7 +574,7 @@ screen_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
     uint64_t* rbuf = P.rowbuf + ((size_t)blockIdx.x * TC_BM + rloc) * P.cap;
     uint32_t* hist = hist_all + warp * 256;
     int64_t tt = 0;
-    int ns = 0;        // norm slot (stage, or ring slot) of tile tt, advanced without dividing
+    int ns = 0;        // norm ring slot of tile tt, advanced without dividing
     uint32_t nph = 0;  // its phase
     bool ok = true;
     for (int64_t rb = blockIdx.x; rb < nrb && ok; rb += gridDim.x) {
@@ -753,10 +589,9 @@ screen_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
         ok = mbar_wait_warp(&t_full[b], (uint32_t)((tt >> TC_NBUF_LOG) & 1), abort_flag, P.status);
         if (!ok) break;
         tc_fence_after();
-        // the tile's column norms: the producer's copy (with the B stage, or into the ring
-        // slot) is complete; the stage cannot be refilled before this warp releases it
-        ok = KSTREAM ? mbar_wait_warp(&n_full[ns], nph, abort_flag, P.status)
-                     : mbar_wait_warp(&b_full[ns], nph, abort_flag, P.status);
+        // the tile's column norms: the producer's copy into the ring slot is complete; the slot
+        // cannot be refilled before this warp releases it
+        ok = mbar_wait_warp(&n_full[ns], nph, abort_flag, P.status);
         if (!ok) break;
         const int64_t c0 = (int64_t)t * TC_BN;
         const bool edge = (c0 + TC_BN > P.n) || (P.self_excl && row >= c0 && row < c0 + TC_BN);
@@ -775,10 +610,10 @@ screen_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
           process_chunk<DUMP>(r, c0 + ch * 32, edge, live, row, P,
                               smem_u32(sNB + ns * TC_BN + ch * 32), thr, cnt, rbuf, dump);
         }
-        // the norms of this slot (stage) are no longer needed: release it to the producer
+        // the norms of this slot are no longer needed: release it to the producer
         __syncwarp();
-        if (lane == 0) mbar_arrive(KSTREAM ? &n_empty[ns] : &b_empty[ns]);
-        if (++ns == (KSTREAM ? TC_NR : P.nst)) {
+        if (lane == 0) mbar_arrive(&n_empty[ns]);
+        if (++ns == TC_NR) {
           ns = 0;
           nph ^= 1u;
         }
@@ -869,8 +704,6 @@ cudaError_t launch_wait_probe(uint32_t* status, const uint32_t* never_set, cudaS
 }
 
 // ---- host side ---------------------------------------------------------------------------------
-// Rows up to 192 wide keep the A tile resident; wider rows stream A and B in K chunks.
-constexpr int TC_KRES_MAX = 192;
 constexpr int TC_KPAD_MAX = 4096;
 
 bool tc_screen_supported(int d, bool) { return d >= 1 && ((d + 63) / 64) * 64 <= TC_KPAD_MAX; }
@@ -915,8 +748,8 @@ static bool make_map(CUtensorMap* map, const void* base, int64_t rows, int kpad,
 static size_t sync_counter_words(int64_t m, int64_t n, int grid) {
   const int64_t nrb = (m + TC_BM - 1) / TC_BM;
   const int64_t waves = (nrb + grid - 1) / grid;
-  const int64_t ntiles = (n + TC_BN - 1) / TC_BN;
-  const int64_t checkpoints = waves * ntiles / TC_SYNC_K + 2;
+  // a window is at most TC_SYNC_COLS columns and at least TC_SYNC_COLS - 128
+  const int64_t checkpoints = waves * (n + 128) / (TC_SYNC_COLS - 128) + 3;
   return (size_t)((checkpoints + 1) / 2);
 }
 
@@ -931,10 +764,10 @@ static uint32_t make_idesc(bool fp16) {
   return d;
 }
 
-template <int CPL, bool DUMP, bool KSTREAM>
+template <int CPL, bool DUMP>
 static cudaError_t launch_t(const CUtensorMap& ma, const CUtensorMap& mb, const TcParams& p,
                            size_t smem, int grid, cudaStream_t s, float* dump) {
-  cudaError_t e = cudaFuncSetAttribute(screen_tc_kernel<CPL, DUMP, KSTREAM>,
+  cudaError_t e = cudaFuncSetAttribute(screen_tc_kernel<CPL, DUMP>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   // cooperative when the producers wait for one another (boundedly): every CTA resident at once
@@ -949,22 +782,16 @@ static cudaError_t launch_t(const CUtensorMap& ma, const CUtensorMap& mb, const 
   cfg.attrs = attr;
   cfg.numAttrs = p.sync ? 1 : 0;
   count_launch();
-  e = cudaLaunchKernelEx(&cfg, screen_tc_kernel<CPL, DUMP, KSTREAM>, ma, mb, p, dump);
+  e = cudaLaunchKernelEx(&cfg, screen_tc_kernel<CPL, DUMP>, ma, mb, p, dump);
   if (e == cudaErrorCooperativeLaunchTooLarge) {  // not all resident: plain launch (waits bounded)
     (void)cudaGetLastError();
     cfg.numAttrs = 0;
-    e = cudaLaunchKernelEx(&cfg, screen_tc_kernel<CPL, DUMP, KSTREAM>, ma, mb, p, dump);
+    e = cudaLaunchKernelEx(&cfg, screen_tc_kernel<CPL, DUMP>, ma, mb, p, dump);
   }
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
 
-// Pipeline variants the autotuner times: operand stages (0 = as many as shared memory holds,
-// else that many fewer), row-buffer capacity step (0 = the smallest that fits, 1 = the next),
-// checkpoint lag in windows of 256 tiles.
-struct TcVariant {
-  int stages_less, cap_step, sync_d;
-};
 constexpr TcVariant TC_VARIANTS[] = {{0, 0, 8}, {0, 0, 4}, {0, 0, 16}, {1, 0, 8}, {0, 1, 8}, {2, 0, 8}};
 constexpr int TC_NVARIANTS = (int)(sizeof(TC_VARIANTS) / sizeof(TC_VARIANTS[0]));
 
@@ -977,21 +804,20 @@ static cudaError_t launch_impl(const TcScreenArgs& a, cudaStream_t s, std::strin
     return cudaErrorInvalidValue;
   }
   const TcVariant v = TC_VARIANTS[variant];
+  if (a.res.kt > 0) return launch_screen_res(a, v, variant, s, msg, dump, shape);
   const int kpad = a.kpad;
   if (kpad % 64 != 0 || kpad < 64 || kpad > TC_KPAD_MAX) {
     if (msg) *msg = "kpad must be a multiple of 64 in [64, 4096]; ";
     return cudaErrorInvalidValue;
   }
-  const bool kstream = kpad > TC_KRES_MAX;
   TcParams p{};
   p.m = a.m;
   p.n = a.n;
   p.kpad = kpad;
   p.nkc = kpad / 64;
-  const int a_bytes = kstream ? 0 : TC_BM * kpad * 2;
-  const int stage_bytes = kstream ? (TC_BM + TC_BN) * TC_KC * 2 : TC_BN * kpad * 2;
-  const int fixed = 1024 + TC_MAXST * TC_BN * 4 + 256 + 8 * 256 * 4;  // alignment, norms, barriers, hist
-  const int budget = 220 * 1024 - a_bytes - fixed;
+  const int stage_bytes = (TC_BM + TC_BN) * TC_KC * 2;
+  const int fixed = 1024 + TC_NR * TC_BN * 4 + 256 + 8 * 256 * 4;  // alignment, norms, barriers, hist
+  const int budget = 220 * 1024 - fixed;
   p.nst = std::min(TC_MAXST, budget / stage_bytes) - v.stages_less;
   if (p.nst < 2) {
     if (msg) *msg = "shared memory too small for two operand stages; ";
@@ -1023,7 +849,7 @@ static cudaError_t launch_impl(const TcScreenArgs& a, cudaStream_t s, std::strin
   const int64_t nrb = (a.m + TC_BM - 1) / TC_BM;
   const int grid = (int)std::min<int64_t>(nrb, num_sms());
   // at least ~116 KB so that a single CTA (and its 512 TMEM columns) fits per SM
-  size_t smem = (size_t)fixed + (size_t)a_bytes + (size_t)p.nst * stage_bytes;
+  size_t smem = (size_t)fixed + (size_t)p.nst * stage_bytes;
   smem = std::max<size_t>(smem, 116 * 1024);
   const size_t buf_words = (size_t)grid * TC_BM * p.cap;
   const size_t sync_words = sync_counter_words(a.m, a.n, grid);
@@ -1041,12 +867,8 @@ static cudaError_t launch_impl(const TcScreenArgs& a, cudaStream_t s, std::strin
   cudaError_t e;
 #define CNG_TC(C)                                                                             \
   case C:                                                                                     \
-    if (kstream)                                                                              \
-      e = dump ? launch_t<C, true, true>(ma, mb, p, smem, grid, s, dump)                      \
-               : launch_t<C, false, true>(ma, mb, p, smem, grid, s, dump);                    \
-    else                                                                                      \
-      e = dump ? launch_t<C, true, false>(ma, mb, p, smem, grid, s, dump)                     \
-               : launch_t<C, false, false>(ma, mb, p, smem, grid, s, dump);                   \
+    e = dump ? launch_t<C, true>(ma, mb, p, smem, grid, s, dump)                              \
+             : launch_t<C, false>(ma, mb, p, smem, grid, s, dump);                            \
     break;
   switch (cpl) {
     CNG_TC(12)
@@ -1074,7 +896,7 @@ size_t screen_tc_rowbuf_words(int64_t m, int64_t n, int Lp) {
 // all the columns; smaller problems use variant 0.  The results of a screen never depend on
 // the variant (the lists are certified and reranked the same way).
 struct TunedScreen {
-  int dev, kpad, Lp, fp16, self, nlog;
+  int dev, kpad, kt, Lp, fp16, self, nlog;
   int variant;
 };
 static std::mutex g_tc_mu;
@@ -1093,11 +915,11 @@ static cudaError_t tune_variant(const TcScreenArgs& a, cudaStream_t s, std::stri
   if (a.m < 4 * sample) return cudaSuccess;  // small problems: the default variant
   int dev = 0;
   cudaGetDevice(&dev);
-  const TunedScreen key{dev, a.kpad, a.Lp, a.fp16, a.self_excl, tune_key_nlog(a.n), 0};
+  const TunedScreen key{dev, a.kpad, a.res.kt, a.Lp, a.fp16, a.self_excl, tune_key_nlog(a.n), 0};
   {
     std::lock_guard<std::mutex> lk(g_tc_mu);
     for (const auto& t : g_tc_tuned)
-      if (t.dev == key.dev && t.kpad == key.kpad && t.Lp == key.Lp && t.fp16 == key.fp16 &&
+      if (t.dev == key.dev && t.kpad == key.kpad && t.kt == key.kt && t.Lp == key.Lp && t.fp16 == key.fp16 &&
           t.self == key.self && t.nlog == key.nlog) {
         *chosen = t.variant;
         return cudaSuccess;
@@ -1116,7 +938,7 @@ static cudaError_t tune_variant(const TcScreenArgs& a, cudaStream_t s, std::stri
     TcScreenArgs t = a;
     const int64_t off = (a.m / 2 / TC_BM) * TC_BM;
     t.row_off = std::min<int64_t>(off, (a.m - sample) / TC_BM * TC_BM);
-    t.A = static_cast<const char*>(a.A) + (size_t)t.row_off * a.kpad * 2;
+    if (a.res.kt == 0) t.A = static_cast<const char*>(a.A) + (size_t)t.row_off * a.kpad * 2;
     t.m = sample;
     t.self_excl = 0;
     t.perm = nullptr;

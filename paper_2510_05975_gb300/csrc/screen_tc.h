@@ -9,7 +9,29 @@
 
 namespace cng {
 
+// Rows of up to 250 coordinates are screened from prepared tile images (k_screen_res.cu): operand
+// width kt (the coordinates and RES_AUX norm pieces, rounded up to 16) and column tile bn.
+constexpr int RES_AUX = 6;
+constexpr int RES_PARTS = 4;                                // parts of the sampled column order
+constexpr float RES_NORM_MAX = 4.f * 65504.f * 32768.f;     // largest ||y_b||^2 / 2 the pieces hold
+struct ResShape {
+  int d = 0, kt = 0, bn = 0;
+};
+// The shape for d coordinates and a largest squared operand norm, or false if not supported.
+bool res_shape(int d, float nbmax, ResShape* r);
+size_t res_image_bytes(const ResShape& r, int64_t rows);
+// out = tile image of xi[perm[p]] (perm null: xi[p]), p < rows; xi: [.][kpad] 16-bit operands with
+// squared norms nb.
+cudaError_t launch_tile_image(const ResShape& r, bool fp16, const void* xi, int kpad, const float* nb,
+                              const int32_t* perm, int64_t rows, void* out, cudaStream_t s);
+
 struct TcScreenArgs {
+  // res.kt > 0: A and B are tile images (nb unused), columns in a sampled order: column position p
+  // is point col_perm[p] and the first part_count[0] positions are the first part, and so on
+  ResShape res;
+  const int32_t* col_perm = nullptr;
+  const int32_t* col_pos = nullptr;  // its inverse (self_excl): the column position of a point
+  int64_t part_count[RES_PARTS] = {0, 0, 0, 0};
   const void* A;      // rows   [m][kpad] bf16 (fp16 when fp16 != 0), zero padded
   const void* B;      // columns [n][kpad]
   int64_t m, n;
@@ -38,6 +60,14 @@ struct TcShape {
   int variant, stages, cap, sync_d;
 };
 int screen_tc_variants();
+// Pipeline variants the autotuner times: operand stages (0 = as many as shared memory holds,
+// else that many fewer), row-buffer capacity step (0 = the smallest that fits, 1 = the next),
+// checkpoint lag in windows of 32,768 columns.
+struct TcVariant {
+  int stages_less, cap_step, sync_d;
+};
+cudaError_t launch_screen_res(const TcScreenArgs& a, const TcVariant& v, int variant, cudaStream_t s,
+                              std::string* msg, float* dump, TcShape* shape);
 // The autotuned variant for a's shape (timing the variants on first use; synchronises `s`).
 cudaError_t launch_screen_tc_tune(const TcScreenArgs& a, cudaStream_t s, std::string* msg, int* variant);
 
