@@ -987,7 +987,8 @@ extern "C" cng_status cng_build(const void* points, int32_t dtype, int64_t n, in
       sa.dists = rdist;
       sa.tot = sc_tot;
       sa.status = sc_status;
-      SearchPlan plan;  // stored points are exact queries: nothing is deferred
+      sa.defer = rp;  // rp is written after the searches
+      SearchPlan plan;
       if (!search_plan(sa, 4, 1024, &plan))
         return fail(CNG_E_UNSUPPORTED, "connectivity search shape does not fit");
       CK(cudaMemsetAsync(sc_counter, 0, SEARCH_COUNTER_INTS * sizeof(int), s));

@@ -69,6 +69,52 @@ CNG_DEV double canon_dist(const TA* x, const TB* y, int d) {
   return __dsqrt_rn(canon_sqdist(x, y, d));
 }
 
+// ---- the canonical squared distance to within DD_EPS, on the FP32 pipe ---------------------------
+// FP64 arithmetic runs at 1/64 of the FP32 rate here (a warp instruction holds the SM's FP64 pipe
+// for 16 cycles), so near-ties are first decided with pairs of FP32 numbers: every difference is
+// split exactly (two-sum), every square has its rounding error (fma) and the cross term of the
+// difference's low part, and the sums carry their rounding errors.  With n = ceil(d / 32) terms per
+// lane, the neglected parts (the low parts' squares, and the FP32 rounding of the error sums, each
+// at most n 2^-24 of the total) stay below (n + 6)^2 2^-48 <= 2^-33 for d <= 4096; DD_EPS leaves a
+// factor 4 on that, the canonical sum's own error (d 2^-53) included.  All lanes take part; every
+// lane gets the value, NaN if it is outside the range in which the bound holds (underflowing
+// squares, overflow, zero): then, and where two values lie within DD_EPS, FP64 decides.
+constexpr double DD_EPS = 4.656612873077393e-10;  // 2^-31
+
+CNG_DEV void two_sum(float a, float b, float& s, float& e) {
+  s = __fadd_rn(a, b);
+  const float z = __fsub_rn(s, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z));
+}
+
+template <typename TA, typename TB>
+CNG_DEV double warp_sqdist_dd(const TA* x, const TB* y, int d, int lane) {
+  float hi = 0.f, lo = 0.f;
+#pragma unroll 2
+  for (int i = lane; i < d; i += 32) {
+    float t, te, s, e;
+    two_sum(to_f(x[i]), -to_f(y[i]), t, te);
+    const float p = __fmul_rn(t, t);
+    const float pe = __fmaf_rn(__fadd_rn(t, t), te, __fmaf_rn(t, t, -p));
+    two_sum(hi, p, s, e);
+    hi = s;
+    lo = __fadd_rn(lo, __fadd_rn(e, pe));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float h2 = __shfl_xor_sync(FULL, hi, o), l2 = __shfl_xor_sync(FULL, lo, o);
+    float s, e;
+    two_sum(fmaxf(hi, h2), fminf(hi, h2), s, e);  // the same sum in both lanes
+    hi = s;
+    lo = __fadd_rn(__fadd_rn(fmaxf(lo, l2), fminf(lo, l2)), e);
+  }
+  const double v = (double)hi + (double)lo;
+  return v >= 1e-25 && v <= 1e30 ? v : __longlong_as_double(0x7ff8000000000000ll);
+}
+
+// Whether two values of warp_sqdist_dd leave the canonical order open.
+CNG_DEV bool dd_open(double a, double b) { return !(fabs(a - b) > DD_EPS * fmax(fabs(a), fabs(b))); }
+
 // Def. 2 / Eq. 1 in double: prunes iff Dpu > alpha * Duv + t, t = (alpha + 1) * tau.
 CNG_DEV bool rule64(double Dpu, double Duv, double alpha, double t) {
   double rhs = __dadd_rn(__dmul_rn(alpha, Duv), t);

@@ -439,9 +439,11 @@ CNG_DEV void warp_bitonic(uint64_t* a, int P2, int lane) {
 // Re-sort, by the canonical (D, id) order, every run of neighbours in keys[0..cnt) whose FP32
 // squared distances are pairwise near-tied and that starts before position `upto`.  `row` is
 // the stored row vector (exact values).  Runs are gathered in batches (up to 32 runs, RR_RUN
-// members); the canonical distances of a batch's members are computed in parallel, one per
-// lane, then lane 0 insertion-sorts each run.  rdesc: [3][32] ints of warp scratch (run start,
-// length, offset in d64).  Returns the number of runs re-decided.
+// members); the members' squared distances are computed to within DD_EPS by the whole warp, one
+// after the other, and lane 0 insertion-sorts each run; only if two of a run lie within DD_EPS are
+// the batch's canonical FP64 distances taken, one per lane, and the runs sorted by those.  rdesc:
+// [3][32] ints of warp scratch (run start, length, offset in d64).  Returns the number of runs
+// re-decided.
 template <typename T>
 CNG_DEV int fix_runs_warp(uint64_t* keys, int cnt, int upto, const T* __restrict__ row,
                           const T* __restrict__ Xc, int dpad, int d, float band, double* d64,
@@ -483,32 +485,46 @@ CNG_DEV int fix_runs_warp(uint64_t* keys, int cnt, int upto, const T* __restrict
     }
     if (nb == 0) break;
     __syncwarp();
-    for (int m = lane; m < total; m += 32) {
-      int k = 0;
-      while (k + 1 < nb && rdesc[64 + k + 1] <= m) ++k;
-      const int pos = rdesc[k] + (m - rdesc[64 + k]);
-      d64[m] = canon_dist(row, Xc + (int64_t)key_id(keys[pos]) * dpad, d);
-    }
+    for (int k = 0; k < nb; ++k)
+      for (int m = 0; m < rdesc[32 + k]; ++m) {
+        const double v = warp_sqdist_dd(row, Xc + (int64_t)key_id(keys[rdesc[k] + m]) * dpad, d, lane);
+        if (lane == 0) d64[rdesc[64 + k] + m] = v;
+      }
     __syncwarp();
-    if (lane == 0) {  // insertion sort of each run by (d64, id)
-      for (int k = 0; k < nb; ++k) {
-        const int s = rdesc[k], len = rdesc[32 + k];
-        double* dd = d64 + rdesc[64 + k];
-        for (int a = 1; a < len; ++a) {
-          double dv = dd[a];
-          uint64_t kv = keys[s + a];
-          int b = a - 1;
-          while (b >= 0 && (dd[b] > dv || (dd[b] == dv && key_id(keys[s + b]) > key_id(kv)))) {
-            dd[b + 1] = dd[b];
-            keys[s + b + 1] = keys[s + b];
-            --b;
+    for (int canon = 0; canon < 2; ++canon) {
+      if (canon) {
+        for (int m = lane; m < total; m += 32) {
+          int k = 0;
+          while (k + 1 < nb && rdesc[64 + k + 1] <= m) ++k;
+          const int pos = rdesc[k] + (m - rdesc[64 + k]);
+          d64[m] = canon_dist(row, Xc + (int64_t)key_id(keys[pos]) * dpad, d);
+        }
+        __syncwarp();
+      }
+      bool open = false;
+      if (lane == 0) {  // insertion sort of each run by (d64, id)
+        for (int k = 0; k < nb; ++k) {
+          const int s = rdesc[k], len = rdesc[32 + k];
+          double* dd = d64 + rdesc[64 + k];
+          for (int a = 1; a < len; ++a) {
+            double dv = dd[a];
+            uint64_t kv = keys[s + a];
+            int b = a - 1;
+            while (b >= 0 && (dd[b] > dv || (dd[b] == dv && key_id(keys[s + b]) > key_id(kv)))) {
+              dd[b + 1] = dd[b];
+              keys[s + b + 1] = keys[s + b];
+              --b;
+            }
+            dd[b + 1] = dv;
+            keys[s + b + 1] = kv;
           }
-          dd[b + 1] = dv;
-          keys[s + b + 1] = kv;
+          if (!canon)
+            for (int a = 1; a < len; ++a) open |= dd_open(dd[a - 1], dd[a]);
         }
       }
+      __syncwarp();
+      if (!__any_sync(FULL, open)) break;
     }
-    __syncwarp();
     runs += nb;
   }
   return runs;

@@ -1,9 +1,10 @@
 // k_search.cu -- batched beam search of Alg. 1 (K7), general kernel, sm_103a.
 //
 // One persistent launch serves the batch: each warp takes the next query from an atomic
-// counter and runs Alg. 1 to completion; queries of any length share the launch.  On data with
-// exact 8-bit rows the register-queue kernel (k_search_fast.cu) runs first and this kernel only
-// serves the queries it deferred (non-integer or out-of-range coordinates).
+// counter and runs Alg. 1 to completion; queries of any length share the launch.  With row strides
+// up to 96 a register-queue kernel (k_search_fast.cu on exact 8-bit rows, else k_search_float.cu)
+// runs first and this kernel only serves the queries it deferred (non-integer or out-of-range
+// coordinates on 8-bit data, near-ties whose FP32 roundings do not settle them).
 //
 // Per warp (shared memory):
 //   Q   sorted queue of <= L entries: key = (FP32 squared distance, id), an explored flag,
@@ -531,14 +532,19 @@ bool search_plan(SearchArgs& a, int wpb, int hash_slots, SearchPlan* p) {
   a.hash_slots = hash_slots;
   a.warp_smem = search_warp_smem(a.dpad, a.L, hash_slots);
   a.warp_smem_fast = 0;
-  // the register-queue kernel: exact data with 8-bit rows, L <= 256, and row stride <= 96
+  // a register-queue kernel: L <= 256 and row stride <= 96; the 8-bit one for exact data with
+  // 8-bit rows.  It needs the list of deferred queries.
   int qs = 0;
-  if (a.U && a.exact && a.dtype == CNG_F32 && a.R <= SQ_ROWSLOTS * 32 && a.k <= a.L)
+  if (a.defer && a.R <= SQ_ROWSLOTS * 32 && a.k <= a.L)
     qs = a.L <= 32 ? 1 : a.L <= 64 ? 2 : a.L <= 128 ? 4 : a.L <= 256 ? 8 : 0;
+  const bool u8 = a.U && a.exact && a.dtype == CNG_F32;
   if (qs) {
-    a.warp_smem_fast = search_fast_warp_smem(a.u8w, hash_slots);
+    const bool learn = a.model || a.trace_feats;
+    a.warp_smem_fast = u8 ? search_fast_warp_smem(a.u8w, hash_slots) : search_float_warp_smem(a.dpad, hash_slots);
     const size_t sh = (size_t)wpb * a.warp_smem_fast + extra_smem;
-    const int b = sh <= kMaxBlockSmem ? search_fast_blocks_per_sm(a.u8w, qs, a.model || a.trace_feats, wpb, sh) : 0;
+    const int b = sh > kMaxBlockSmem ? 0
+                  : u8               ? search_fast_blocks_per_sm(a.u8w, qs, learn, wpb, sh)
+                                     : search_float_blocks_per_sm(a.dtype, qs, learn, wpb, sh);
     if (b < 1) return false;
     p->grid = num_sms() * b;
     p->fast_qs = qs;
@@ -564,7 +570,8 @@ bool search_plan(SearchArgs& a, int wpb, int hash_slots, SearchPlan* p) {
 
 cudaError_t launch_search(const SearchArgs& a, const SearchPlan& p, cudaStream_t s) {
   if (p.fast_qs == 0) return launch_search_general(a, p.wpb, p.grid, s);
-  cudaError_t e = launch_search_fast(a, p.fast_qs, p.wpb, p.grid, s);
+  cudaError_t e = a.U && a.exact && a.dtype == CNG_F32 ? launch_search_fast(a, p.fast_qs, p.wpb, p.grid, s)
+                                                        : launch_search_float(a, p.fast_qs, p.wpb, p.grid, s);
   if (e != cudaSuccess) return e;
   SearchArgs g = a;
   g.qlist = a.defer;

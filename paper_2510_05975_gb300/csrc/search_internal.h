@@ -61,10 +61,10 @@ struct SearchArgs {
 
 constexpr int SEARCH_COUNTER_INTS = 4;
 
-// Launch shape of one batched search.  fast_qs > 0: the register-queue kernel (queue of up to
-// 32 * fast_qs entries in registers; data with 8-bit rows) runs first on `grid` blocks, then the
-// general kernel on `grid_defer` blocks for the deferred queries; fast_qs == 0: the general
-// kernel alone on `grid` blocks.
+// Launch shape of one batched search.  fast_qs > 0: a register-queue kernel (queue of up to
+// 32 * fast_qs entries in registers; k_search_fast.cu for data with 8-bit rows, else
+// k_search_float.cu) runs first on `grid` blocks, then the general kernel on `grid_defer` blocks for
+// the deferred queries; fast_qs == 0: the general kernel alone on `grid` blocks.
 struct SearchPlan {
   int wpb = 0;
   int grid = 0;
@@ -95,6 +95,9 @@ cudaError_t launch_query_check(const float* Q, int64_t nq, int d, float vmin, fl
 int search_blocks_per_sm(int dtype, int u8w, int warps_per_block, size_t smem);
 int search_fast_blocks_per_sm(int u8w, int qs, bool learn, int warps_per_block, size_t smem);
 size_t search_fast_warp_smem(int u8w, int hash_slots);
+int search_float_blocks_per_sm(int dtype, int qs, bool learn, int warps_per_block, size_t smem);
+size_t search_float_warp_smem(int dpad, int hash_slots);
+cudaError_t launch_search_float(const SearchArgs& a, int qs, int warps_per_block, int grid, cudaStream_t s);
 cudaError_t launch_search_general(const SearchArgs& a, int warps_per_block, int grid, cudaStream_t s);
 cudaError_t launch_search_fast(const SearchArgs& a, int qs, int warps_per_block, int grid, cudaStream_t s);
 
