@@ -897,6 +897,10 @@ extern "C" cng_status cng_build(const void* points, int32_t dtype, int64_t n, in
     CK(pool.alloc(&ms.mdist, (size_t)n * ms.stride));
     CK(pool.alloc(&ms.mlen, (size_t)n));
     CK(pool.alloc(&ms.rlist, (size_t)n));
+    if (half_norms) {  // the norms of the FP16 prune serve the re-prune too
+      CK(pool.alloc(&ms.slist, (size_t)n));
+      ms.nrm = half_norms;
+    }
   }
   CK(launch_merge(pr.xs, dtype, n, d, dpad, fwd, fdeg, off, inl, P.alpha, P.tau, ag, R, band, exact, adj,
                   deg, Rs, ctr, big_list, u8, u8w, ms, s));

@@ -41,18 +41,23 @@ struct Counters {
   int max_indeg;
   int nmid;        // 8-bit merge: nodes deferred from the 128-entry to the 256-entry pass
   unsigned long long alpha_steps;  // adaptive pruning: sum over phase-2 points of the alpha step
-  int nre;         // 8-bit merge: nodes listed for the pipelined Gram re-prune
+  int nre;         // merged sets listed for the re-prune (Gram tile of 8-bit rows, all-pairs kernel)
+  int nsmall;      // FP16 merge: sets of up to 128 listed for the Gram tile
 };
 
 // Scratch of the merge's re-prune by the Gram-tile / all-pairs kernels: merged lists in (D, id)
 // order of up to `stride` entries per node ([n][stride] ids and FP32 distances; 128 for 8-bit
-// rows, 256 for float rows), their lengths and the listed nodes.  All null: not used.
+// rows, 256 for float rows), their lengths and the listed nodes; with slist and nrm (FP16 rows: the
+// points' |x|^2) the sets of up to 128 entries are listed in slist for the Gram tile.  All null: not
+// used.
 struct MergeScratch {
   int32_t* mlist;
   float* mdist;
   int32_t* mlen;
   int32_t* rlist;
   int stride;
+  int32_t* slist;
+  const float* nrm;
 };
 
 // Alg. 4 grid of adaptive pruning: alpha_i = alpha0 + i * dalpha, i = 0 .. imax (imax < 0:

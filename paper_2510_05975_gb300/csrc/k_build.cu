@@ -13,6 +13,7 @@
 #include "launch_count.h"
 #include "cng_internal.h"
 #include "device_common.cuh"
+#include "row_warp.cuh"
 
 namespace cng {
 
@@ -418,117 +419,7 @@ cudaError_t launch_knn_simt(const void* xr, int64_t m, const void* xc, int64_t n
 // ============================================================================================
 constexpr int RR_WARPS = 4;
 constexpr int RR_P2 = 512;      // max screened list (power of two)
-constexpr int RR_RUN = 256;     // longest near-tie run re-sorted in FP64
 constexpr int RR_G = 8;         // lanes per distance
-
-CNG_DEV void warp_bitonic(uint64_t* a, int P2, int lane) {
-  for (int k = 2; k <= P2; k <<= 1)
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int i = lane; i < P2; i += 32) {
-        int ixj = i ^ j;
-        if (ixj > i) {
-          uint64_t x = a[i], y = a[ixj];
-          bool up = (i & k) == 0;
-          if ((x > y) == up) { a[i] = y; a[ixj] = x; }
-        }
-      }
-      __syncwarp();
-    }
-}
-
-// Re-sort, by the canonical (D, id) order, every run of neighbours in keys[0..cnt) whose FP32
-// squared distances are pairwise near-tied and that starts before position `upto`.  `row` is
-// the stored row vector (exact values).  Runs are gathered in batches (up to 32 runs, RR_RUN
-// members); the members' squared distances are computed to within DD_EPS by the whole warp, one
-// after the other, and lane 0 insertion-sorts each run; only if two of a run lie within DD_EPS are
-// the batch's canonical FP64 distances taken, one per lane, and the runs sorted by those.  rdesc:
-// [3][32] ints of warp scratch (run start, length, offset in d64).  Returns the number of runs
-// re-decided.
-template <typename T>
-CNG_DEV int fix_runs_warp(uint64_t* keys, int cnt, int upto, const T* __restrict__ row,
-                          const T* __restrict__ Xc, int dpad, int d, float band, double* d64,
-                          int* rdesc, int lane, uint32_t* status) {
-  int runs = 0;
-  int i = 0;
-  while (i < upto && i + 1 < cnt) {
-    int nb = 0, total = 0;
-    while (nb < 32 && i < upto && i + 1 < cnt) {
-      // the next run start >= i (lane-parallel scan, 32 pairs at a time)
-      int s = -1;
-      for (int b = i; b < upto && b + 1 < cnt && s < 0; b += 32) {
-        int t = b + lane;
-        bool nt = t < upto && t + 1 < cnt && near_tie(key_dist(keys[t]), key_dist(keys[t + 1]), band);
-        unsigned bal = __ballot_sync(FULL, nt);
-        if (bal) s = b + __ffs(bal) - 1;
-      }
-      if (s < 0) {
-        i = upto;
-        break;
-      }
-      int e = s + 1;  // run is [s, e]
-      while (e + 1 < cnt && near_tie(key_dist(keys[e]), key_dist(keys[e + 1]), band)) ++e;
-      int len = e - s + 1;
-      if (len > RR_RUN) {
-        if (lane == 0) set_status(status, ST_OVF_RUN);
-        len = RR_RUN;
-        e = s + len - 1;
-      }
-      if (total + len > RR_RUN) break;  // this run opens the next batch
-      if (lane == 0) {
-        rdesc[nb] = s;
-        rdesc[32 + nb] = len;
-        rdesc[64 + nb] = total;
-      }
-      total += len;
-      ++nb;
-      i = e + 1;
-    }
-    if (nb == 0) break;
-    __syncwarp();
-    for (int k = 0; k < nb; ++k)
-      for (int m = 0; m < rdesc[32 + k]; ++m) {
-        const double v = warp_sqdist_dd(row, Xc + (int64_t)key_id(keys[rdesc[k] + m]) * dpad, d, lane);
-        if (lane == 0) d64[rdesc[64 + k] + m] = v;
-      }
-    __syncwarp();
-    for (int canon = 0; canon < 2; ++canon) {
-      if (canon) {
-        for (int m = lane; m < total; m += 32) {
-          int k = 0;
-          while (k + 1 < nb && rdesc[64 + k + 1] <= m) ++k;
-          const int pos = rdesc[k] + (m - rdesc[64 + k]);
-          d64[m] = canon_dist(row, Xc + (int64_t)key_id(keys[pos]) * dpad, d);
-        }
-        __syncwarp();
-      }
-      bool open = false;
-      if (lane == 0) {  // insertion sort of each run by (d64, id)
-        for (int k = 0; k < nb; ++k) {
-          const int s = rdesc[k], len = rdesc[32 + k];
-          double* dd = d64 + rdesc[64 + k];
-          for (int a = 1; a < len; ++a) {
-            double dv = dd[a];
-            uint64_t kv = keys[s + a];
-            int b = a - 1;
-            while (b >= 0 && (dd[b] > dv || (dd[b] == dv && key_id(keys[s + b]) > key_id(kv)))) {
-              dd[b + 1] = dd[b];
-              keys[s + b + 1] = keys[s + b];
-              --b;
-            }
-            dd[b + 1] = dv;
-            keys[s + b + 1] = kv;
-          }
-          if (!canon)
-            for (int a = 1; a < len; ++a) open |= dd_open(dd[a - 1], dd[a]);
-        }
-      }
-      __syncwarp();
-      if (!__any_sync(FULL, open)) break;
-    }
-    runs += nb;
-  }
-  return runs;
-}
 
 // Squared FP32 distances of the query slice held in registers (lane l holds float4 chunks
 // l, l + 32, ..., NQ of them) to two stored rows read by the whole warp (coalesced 16-byte

@@ -15,6 +15,7 @@
 #include "launch_count.h"
 #include "cng_internal.h"
 #include "device_common.cuh"
+#include "row_warp.cuh"
 #include "prune_rule.cuh"
 #include "prune_tc.h"
 
@@ -832,56 +833,89 @@ CNG_DEV int merge_node(const T* __restrict__ Xs, int d, int dpad, int64_t p,
             i = e + 1;
             continue;
           }
-          for (int t = lane; t < len; t += 32) {
-            rid[t] = key_id(ar.keys[s + t]);
-            d64[t] = canon_dist(Xs + p * dpad, Xs + (int64_t)rid[t] * dpad, d);
-          }
-          __syncwarp();
-          if (lane == 0) {  // insertion sort of the run by (D, id)
-            for (int a = 1; a < len; ++a) {
-              double dv = d64[a];
-              int32_t iv = rid[a];
-              uint64_t kv = ar.keys[s + a];
-              int b = a - 1;
-              while (b >= 0 && (d64[b] > dv || (d64[b] == dv && rid[b] > iv))) {
-                d64[b + 1] = d64[b];
-                rid[b + 1] = rid[b];
-                ar.keys[s + b + 1] = ar.keys[s + b];
-                --b;
+          // by squared distances to within DD_EPS (the whole warp, member by member); in FP64
+          // only if two of the run lie that close (a lane's FP64 sum takes ~0.4 us a coordinate)
+          for (int canon = 0; canon < 2; ++canon) {
+            if (canon) {
+              for (int t = lane; t < len; t += 32) {
+                rid[t] = key_id(ar.keys[s + t]);
+                d64[t] = canon_dist(Xs + p * dpad, Xs + (int64_t)rid[t] * dpad, d);
               }
-              d64[b + 1] = dv;
-              rid[b + 1] = iv;
-              ar.keys[s + b + 1] = kv;
+            } else {
+              for (int t = 0; t < len; ++t) {
+                const int32_t id = key_id(ar.keys[s + t]);
+                const double v = warp_sqdist_dd(Xs + p * dpad, Xs + (int64_t)id * dpad, d, lane);
+                if (lane == 0) {
+                  rid[t] = id;
+                  d64[t] = v;
+                }
+              }
             }
-            s_qend = max(s_qend, e + 1);
+            __syncwarp();
+            bool open = false;
+            if (lane == 0) {  // insertion sort of the run by (D, id)
+              for (int a = 1; a < len; ++a) {
+                double dv = d64[a];
+                int32_t iv = rid[a];
+                uint64_t kv = ar.keys[s + a];
+                int b = a - 1;
+                while (b >= 0 && (d64[b] > dv || (d64[b] == dv && rid[b] > iv))) {
+                  d64[b + 1] = d64[b];
+                  rid[b + 1] = rid[b];
+                  ar.keys[s + b + 1] = ar.keys[s + b];
+                  --b;
+                }
+                d64[b + 1] = dv;
+                rid[b + 1] = iv;
+                ar.keys[s + b + 1] = kv;
+              }
+              if (!canon)
+                for (int a = 1; a < len; ++a) open |= dd_open(d64[a - 1], d64[a]);
+              s_qend = max(s_qend, e + 1);
+            }
+            __syncwarp();
+            if (!__any_sync(FULL, open)) break;
           }
-          __syncwarp();
           ++ordties;
           i = e + 1;
         }
       }
       __syncthreads();
-      // long runs: canonical distances of the whole run (in the id / dist arrays, free until
-      // they are filled below), then an odd-even transposition sort of the run by (D, id)
+      // long runs: distances of the whole run (in the id / dist arrays, free until they are filled
+      // below), to within DD_EPS first as above, then an odd-even transposition sort of the run by
+      // (D, id)
       const int nlr = s_nlr;
       for (int r = 0; r < nlr; ++r) {
         const int s0 = s_lr_start[r], len = s_lr_len[r];
         double* D = reinterpret_cast<double*>(ar.ids);  // ids and dist: 8 bytes per entry, contiguous
-        for (int t = tid; t < len; t += PR_THREADS)
-          D[t] = canon_dist(Xs + p * dpad, Xs + (int64_t)key_id(ar.keys[s0 + t]) * dpad, d);
-        __syncthreads();
-        for (int ph = 0; ph < len; ++ph) {
-          for (int t = 2 * tid + (ph & 1); t + 1 < len; t += 2 * PR_THREADS) {
-            const uint64_t ka = ar.keys[s0 + t], kb = ar.keys[s0 + t + 1];
-            if (D[t + 1] < D[t] || (D[t + 1] == D[t] && key_id(kb) < key_id(ka))) {
-              const double tdv = D[t];
-              D[t] = D[t + 1];
-              D[t + 1] = tdv;
-              ar.keys[s0 + t] = kb;
-              ar.keys[s0 + t + 1] = ka;
+        for (int canon = 0; canon < 2; ++canon) {
+          if (canon) {
+            for (int t = tid; t < len; t += PR_THREADS)
+              D[t] = canon_dist(Xs + p * dpad, Xs + (int64_t)key_id(ar.keys[s0 + t]) * dpad, d);
+          } else {
+            for (int t = warp; t < len; t += PR_THREADS / 32) {
+              const double v = warp_sqdist_dd(Xs + p * dpad, Xs + (int64_t)key_id(ar.keys[s0 + t]) * dpad, d, lane);
+              if (lane == 0) D[t] = v;
             }
           }
           __syncthreads();
+          for (int ph = 0; ph < len; ++ph) {
+            for (int t = 2 * tid + (ph & 1); t + 1 < len; t += 2 * PR_THREADS) {
+              const uint64_t ka = ar.keys[s0 + t], kb = ar.keys[s0 + t + 1];
+              if (D[t + 1] < D[t] || (D[t + 1] == D[t] && key_id(kb) < key_id(ka))) {
+                const double tdv = D[t];
+                D[t] = D[t + 1];
+                D[t + 1] = tdv;
+                ar.keys[s0 + t] = kb;
+                ar.keys[s0 + t + 1] = ka;
+              }
+            }
+            __syncthreads();
+          }
+          bool open = false;
+          if (!canon)
+            for (int t = tid; t + 1 < len; t += PR_THREADS) open |= dd_open(D[t], D[t + 1]);
+          if (!__syncthreads_or(open)) break;
         }
       }
       from = s_next;
@@ -959,7 +993,8 @@ merge_kernel(const T* __restrict__ Xs, int64_t n, int d, int dpad, const int32_t
              const int32_t* __restrict__ fdeg, const int64_t* __restrict__ off,
              const int32_t* __restrict__ inl, RuleArgs ra, int exact, int32_t* __restrict__ adj,
              int32_t* __restrict__ deg, Counters* ctr, int32_t* __restrict__ big_list,
-             unsigned char* __restrict__ big_scratch, int big_cap, MergeScratch ms) {
+             unsigned char* __restrict__ big_scratch, int big_cap, MergeScratch ms,
+             const int32_t* __restrict__ mid_list) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_nv;
   PruneSmem sm;
@@ -988,9 +1023,10 @@ merge_kernel(const T* __restrict__ Xs, int64_t n, int d, int dpad, const int32_t
   sm.stage = reinterpret_cast<float*>(ptr);
   const int tid = threadIdx.x, lane = tid & 31;
   unsigned long long ties = 0, ordties = 0, repruned = 0, edges = 0, maxlist = 0;
-  const int64_t count = BIG ? (int64_t)ctr->nbig : n;
+  // every node, the nodes listed by merge_lists_kernel, or (BIG) those above the shared capacity
+  const int64_t count = BIG ? (int64_t)ctr->nbig : (mid_list ? (int64_t)ctr->nmid : n);
   for (int64_t q = blockIdx.x; q < count; q += gridDim.x) {
-    const int64_t p = BIG ? (int64_t)big_list[q] : q;
+    const int64_t p = BIG ? (int64_t)big_list[q] : (mid_list ? (int64_t)mid_list[q] : q);
     const int nf = fdeg[p];
     const int64_t i0 = off[p];
     const int nin = (int)(off[p + 1] - i0);
@@ -1013,6 +1049,115 @@ merge_kernel(const T* __restrict__ Xs, int64_t n, int d, int dpad, const int32_t
     if (ordties) atomicAdd(&ctr->order_ties, ordties);
     atomicAdd(&ctr->merge_repruned, repruned);
     atomicAdd(&ctr->edges, edges);
+    atomicMax(&ctr->merge_max_list, maxlist);
+  }
+}
+
+// The merged sets of float rows that the re-prune kernels take (up to ML_CAP entries before
+// duplicates leave): one warp per node gathers V'(p), takes its distances (4 rows per load
+// instruction, 16 in flight) and orders it by (D(p,.), id); sets of at most R entries become rows at
+// once, the others are listed.  Nodes with more entries go to mid_list for merge_kernel.  Bound by the
+// rows' gathers; a CTA per node with its barriers and 100 KB of shared memory (merge_kernel) kept 16
+// warps on an SM, this 32 or more.  1M x 96 (R = 48): 45 -> 16 ms; 1M x 128 FP16: 31 -> 11 ms.
+constexpr int ML_CAP = 256;
+constexpr int ML_WARPS = 4;
+constexpr size_t ml_warp_bytes(int dpad) {
+  return ML_CAP * 8 + RR_RUN * 8 + 96 * 4 + 64 * 4 + (size_t)dpad * 4;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(ML_WARPS * 32)
+merge_lists_kernel(const T* __restrict__ Xs, int64_t n, int d, int dpad, const int32_t* __restrict__ fwd,
+                   const int32_t* __restrict__ fdeg, const int64_t* __restrict__ off,
+                   const int32_t* __restrict__ inl, RuleArgs ra, int exact, int32_t* __restrict__ adj,
+                   int32_t* __restrict__ deg, Counters* ctr, int32_t* __restrict__ mid_list,
+                   MergeScratch ms) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned char* base = smem + warp * ml_warp_bytes(dpad);
+  float* pq = reinterpret_cast<float*>(base);
+  uint64_t* keys = reinterpret_cast<uint64_t*>(base + (size_t)dpad * 4);
+  double* d64 = reinterpret_cast<double*>(keys + ML_CAP);
+  int* rdesc = reinterpret_cast<int*>(d64 + RR_RUN);
+  int32_t* f = rdesc + 96;
+  const int g = lane % 8, grp = lane / 8;
+  unsigned long long ordties = 0, edges = 0, maxlist = 0;
+  for (int64_t p = (int64_t)blockIdx.x * ML_WARPS + warp; p < n; p += (int64_t)gridDim.x * ML_WARPS) {
+    const int nf = fdeg[p];
+    const int64_t i0 = off[p];
+    const int nin = (int)(off[p + 1] - i0);
+    maxlist = max(maxlist, (unsigned long long)(nf + nin));
+    if (nf + nin > ML_CAP) {
+      if (lane == 0) mid_list[atomicAdd(&ctr->nmid, 1)] = (int32_t)p;
+      continue;
+    }
+    __syncwarp();
+    for (int i = lane; i < nf; i += 32) {
+      const int32_t u = fwd[p * ra.R + i];
+      f[i] = u;
+      keys[i] = (uint32_t)u;
+    }
+    load_row(pq, Xs + p * dpad, dpad, lane, 32);
+    __syncwarp();
+    int nv = nf;
+    for (int b = 0; b < nin; b += 32) {  // in-neighbours that are not out-neighbours
+      const int32_t u = b + lane < nin ? inl[i0 + b + lane] : -1;
+      bool keep = u >= 0;
+      for (int j = 0; j < nf; ++j) keep = keep && f[j] != u;
+      const unsigned bal = __ballot_sync(FULL, keep);
+      if (keep) keys[nv + __popc(bal & ((1u << lane) - 1))] = (uint32_t)u;
+      nv += __popc(bal);
+    }
+    __syncwarp();
+    for (int b = 0; b < nv; b += 16) {
+      const T* y[4];
+      int32_t id[4];
+      float s[4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const int i = b + 4 * r + grp;
+        id[r] = key_id(keys[i < nv ? i : 0]);  // the id is the low word, before and after packing
+        y[r] = Xs + (int64_t)id[r] * dpad;
+      }
+      part_rows<4>(pq, y, dpad, g, s);
+      __syncwarp();
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        s[r] = group_reduce<8>(s[r]);
+        const int i = b + 4 * r + grp;
+        if (g == 0 && i < nv) keys[i] = pack_key(s[r], id[r]);
+      }
+      __syncwarp();
+    }
+    int P2 = 32;
+    while (P2 < nv) P2 <<= 1;
+    __syncwarp();
+    for (int i = nv + lane; i < P2; i += 32) keys[i] = ~0ull;
+    __syncwarp();
+    warp_bitonic(keys, P2, lane);
+    if (!exact)
+      ordties += fix_runs_warp(keys, nv, nv, Xs + p * dpad, Xs, dpad, d, ra.band, d64, rdesc, lane, &ctr->status);
+    if (nv <= ra.R) {
+      for (int i = lane; i < ra.rs; i += 32) adj[p * ra.rs + i] = i < nv ? key_id(keys[i]) : -1;
+      if (lane == 0) deg[p] = nv;
+      edges += nv;
+    } else {
+      for (int i = lane; i < nv; i += 32) {
+        ms.mlist[p * ms.stride + i] = key_id(keys[i]);
+        ms.mdist[p * ms.stride + i] = sqrtf(key_dist(keys[i]));
+      }
+      if (lane == 0) {
+        ms.mlen[p] = nv;
+        if (ms.slist && nv <= 128)
+          ms.slist[atomicAdd(&ctr->nsmall, 1)] = (int32_t)p;
+        else
+          ms.rlist[atomicAdd(&ctr->nre, 1)] = (int32_t)p;
+      }
+    }
+  }
+  if (lane == 0) {
+    if (ordties) atomicAdd(&ctr->order_ties, ordties);
+    if (edges) atomicAdd(&ctr->edges, edges);
     atomicMax(&ctr->merge_max_list, maxlist);
   }
 }
@@ -1138,11 +1283,23 @@ static cudaError_t merge_t2(const void* xs, int64_t n, int d, int dpad, const in
               (size_t)stage_cap * dpad * 4 + 16;
   cudaFuncSetAttribute(merge_kernel<T, BIG, NS, DL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)sh);
-  count_launch();
   const MergeScratch mk = BIG ? MergeScratch{} : ms;
+  const int32_t* mid_list = nullptr;
+  if (mk.mlist && mk.stride >= ML_CAP) {  // the ordinary nodes, one warp each; the rest is listed
+    const size_t shl = ML_WARPS * ml_warp_bytes(dpad);
+    cudaFuncSetAttribute(merge_lists_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shl);
+    int nb = 1;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, merge_lists_kernel<T>, ML_WARPS * 32, shl);
+    const int gl = (int)std::min<int64_t>((n + ML_WARPS - 1) / ML_WARPS, (int64_t)num_sms() * std::max(nb, 1));
+    mid_list = big_list + n;
+    count_launch();
+    merge_lists_kernel<T><<<gl, ML_WARPS * 32, shl, s>>>((const T*)xs, n, d, dpad, fwd, fdeg, off, inl, ra,
+                                                         exact, adj, deg, ctr, big_list + n, mk);
+  }
+  count_launch();
   merge_kernel<T, BIG, NS, DL><<<grid, PR_THREADS, sh, s>>>((const T*)xs, n, d, dpad, fwd, fdeg, off,
                                                             inl, ra, exact, adj, deg, ctr, big_list,
-                                                            big_scratch, big_cap, mk);
+                                                            big_scratch, big_cap, mk, mid_list);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess && mk.mlist)
     e = launch_merge_pairs(xs, sizeof(T) == 4 ? CNG_F32 : CNG_F16, n, d, dpad, mk, ra, adj, deg, ctr, s);

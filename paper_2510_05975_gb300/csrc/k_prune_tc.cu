@@ -1223,6 +1223,21 @@ cudaError_t launch_prune_pairs(const void* xs, int dtype, int64_t n, int d, int 
 cudaError_t launch_merge_pairs(const void* xs, int dtype, int64_t n, int d, int dpad,
                                const MergeScratch& ms, const RuleArgs& ra, int32_t* adj, int32_t* deg,
                                Counters* ctr, cudaStream_t s) {
+  if (ms.slist) {  // FP16 rows, sets of up to 128: the Gram tile of the prune
+    const GramJob S{ms.mlist, ms.mdist, ms.stride, ms.mlen, 0, ms.slist, &ctr->nsmall, n, adj, ra.rs, deg, 1,
+                    ms.nrm};
+    const __half* X = static_cast<const __half*>(xs);
+    count_launch();
+    if (dpad == 128) {
+      prepare(gram_pipe_kernel<__half, 128, true>);
+      gram_pipe_kernel<__half, 128, true><<<num_sms() * 4, GP_THREADS, GT_SMEM, s>>>(nullptr, X, d, dpad, S, ra, ctr);
+    } else {
+      prepare(gram_pipe_kernel<__half, 64, true>);
+      gram_pipe_kernel<__half, 64, true><<<num_sms() * 4, GP_THREADS, GT_SMEM, s>>>(nullptr, X, d, dpad, S, ra, ctr);
+    }
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
   const GramJob J{ms.mlist, ms.mdist, ms.stride, ms.mlen, 0, ms.rlist, &ctr->nre, n, adj, ra.rs, deg, 1,
                   nullptr};
   return pairs_job(xs, dtype, d, dpad, J, ra, ctr, s);

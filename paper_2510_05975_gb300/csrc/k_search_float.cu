@@ -32,6 +32,7 @@
 #include "launch_count.h"
 #include "cng_internal.h"
 #include "device_common.cuh"
+#include "row_warp.cuh"
 #include "search_internal.h"
 #include "search_device.cuh"
 
@@ -279,86 +280,6 @@ __device__ __noinline__ bool fq_fix(uint64_t* qm, uint64_t drop, const float* qv
   *dec_out = dec;
   *moves_io = moves;
   return settled;
-}
-
-// part_sqdist<8> on NR rows at once, in its order: partial squared distances of rows y[r] (r < NR)
-// for lane g of a group of 8.
-template <int NR>
-CNG_DEV void part_rows(const float* __restrict__ q, const float* const (&y)[NR], int dpad, int g,
-                       float (&p)[NR]) {
-  const float4* q4 = reinterpret_cast<const float4*>(q) + g;
-  const int u = dpad >> 5;  // chunks per lane
-  float s0[NR], s1[NR], s2[NR], s3[NR];
-#pragma unroll
-  for (int r = 0; r < NR; ++r) s0[r] = s1[r] = s2[r] = s3[r] = 0.f;
-  int t = 0;
-  for (; t + 3 < u; t += 4) {
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      float4 x[NR][2];
-#pragma unroll
-      for (int r = 0; r < NR; ++r) {
-        const float4* y4 = reinterpret_cast<const float4*>(y[r]) + g + 8 * t + 16 * h;
-        x[r][0] = __ldg(y4);
-        x[r][1] = __ldg(y4 + 8);
-      }
-      const float4 a0 = q4[8 * t + 16 * h], a1 = q4[8 * t + 16 * h + 8];
-#pragma unroll
-      for (int r = 0; r < NR; ++r) {
-        acc4(a0, x[r][0], h ? s2[r] : s0[r]);
-        acc4(a1, x[r][1], h ? s3[r] : s1[r]);
-      }
-    }
-  }
-#pragma unroll 3
-  for (; t < u; ++t) {
-    float4 x[NR];
-#pragma unroll
-    for (int r = 0; r < NR; ++r) x[r] = __ldg(reinterpret_cast<const float4*>(y[r]) + g + 8 * t);
-    const float4 a = q4[8 * t];
-#pragma unroll
-    for (int r = 0; r < NR; ++r) acc4(a, x[r], s0[r]);
-  }
-#pragma unroll
-  for (int r = 0; r < NR; ++r) p[r] = (s0[r] + s1[r]) + (s2[r] + s3[r]);
-}
-template <int NR>
-CNG_DEV void part_rows(const float* __restrict__ q, const __half* const (&y)[NR], int dpad, int g,
-                       float (&p)[NR]) {
-  const float4* q4 = reinterpret_cast<const float4*>(q) + 2 * g;
-  const int u = dpad >> 6;  // chunks of 8 halves per lane
-  float s0[NR], s1[NR], s2[NR], s3[NR];
-#pragma unroll
-  for (int r = 0; r < NR; ++r) s0[r] = s1[r] = s2[r] = s3[r] = 0.f;
-  int t = 0;
-  for (; t + 1 < u; t += 2) {
-    uint4 x[NR][2];
-#pragma unroll
-    for (int r = 0; r < NR; ++r) {
-      const uint4* y8 = reinterpret_cast<const uint4*>(y[r]) + g + 8 * t;
-      x[r][0] = __ldg(y8);
-      x[r][1] = __ldg(y8 + 8);
-    }
-    const float4 a0 = q4[16 * t], a1 = q4[16 * t + 1], b0 = q4[16 * t + 16], b1 = q4[16 * t + 17];
-#pragma unroll
-    for (int r = 0; r < NR; ++r) {
-      acc4(a0, h8lo(x[r][0]), s0[r]);
-      acc4(a1, h8hi(x[r][0]), s1[r]);
-      acc4(b0, h8lo(x[r][1]), s2[r]);
-      acc4(b1, h8hi(x[r][1]), s3[r]);
-    }
-  }
-  for (; t < u; ++t) {
-    const float4 a0 = q4[16 * t], a1 = q4[16 * t + 1];
-#pragma unroll
-    for (int r = 0; r < NR; ++r) {
-      const uint4 x = __ldg(reinterpret_cast<const uint4*>(y[r]) + g + 8 * t);
-      acc4(a0, h8lo(x), s0[r]);
-      acc4(a1, h8hi(x), s1[r]);
-    }
-  }
-#pragma unroll
-  for (int r = 0; r < NR; ++r) p[r] = (s0[r] + s1[r]) + (s2[r] + s3[r]);
 }
 
 // FP32 squared distances of the query to up to 32 rows (row b named by lane b's v, present when
