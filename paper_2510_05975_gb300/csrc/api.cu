@@ -1893,7 +1893,7 @@ extern "C" cng_status cng_stop_train(const cng_index* cix, const float* train_q,
   CK(cudaStreamSynchronize(s));
   tm.mark();
   if (N < 1) return fail(CNG_E_INVAL, "traces produced no samples");
-  float *X, *y, *part, *ploss, *grad, *loss, *m, *v;
+  float *X, *y, *scratch, *loss, *m, *v;
   double* spart;
   unsigned long long* npos;
   CK(pool.alloc(&X, (size_t)N * 16));
@@ -1901,9 +1901,7 @@ extern "C" cng_status cng_stop_train(const cng_index* cix, const float* train_q,
   CK(pool.alloc(&spart, 64 * 32));
   CK(pool.alloc(&npos, 1));
   const int Bn = (int)std::min<int64_t>(B, N);
-  CK(pool.alloc(&part, (size_t)mlp_parts(Bn) * MLP_NPARAMS));
-  CK(pool.alloc(&ploss, (size_t)mlp_parts(Bn)));
-  CK(pool.alloc(&grad, MLP_NPARAMS));
+  CK(pool.alloc(&scratch, mlp_scratch_floats(Bn)));
   CK(pool.alloc(&loss, 2));
   CK(pool.alloc(&m, MLP_NPARAMS));
   CK(pool.alloc(&v, MLP_NPARAMS));
@@ -1931,8 +1929,7 @@ extern "C" cng_status cng_stop_train(const cng_index* cix, const float* train_q,
   const uint64_t seed = (P.seed ? P.seed : 1) * 0x2545F4914F6CDD1Dull + 7;
   for (int64_t t = 1; t <= steps; ++t) {
     float* lp = (t == 1) ? loss : (t == steps ? loss + 1 : nullptr);
-    CKM(launch_mlp_grad(mdl->P, X, y, N, Bn, seed, t, part, ploss, grad, lp, s));
-    CKM(launch_adam(mdl->P, m, v, grad, t, lr, s));
+    CKM(launch_mlp_step(mdl->P, X, y, N, Bn, seed, t, lr, m, v, scratch, lp, s));
   }
   CKM(launch_pack_model(mdl->P, mdl->mu, mdl->sg, mdl->blk, s));
   tm.mark();
@@ -2008,11 +2005,10 @@ extern "C" cng_status cng_mlp_grad(const float* params, const float* x, const fl
   if (B < 1 || B > (1 << 22)) return fail(CNG_E_INVAL, "B must be in [1, 2^22]");
   cudaStream_t s = (cudaStream_t)stream;
   DevPool pool;
-  float *part, *ploss, *l;
-  CK(pool.alloc(&part, (size_t)mlp_parts((int)B) * MLP_NPARAMS));
-  CK(pool.alloc(&ploss, (size_t)mlp_parts((int)B)));
+  float *scratch, *l;
+  CK(pool.alloc(&scratch, mlp_scratch_floats((int)B)));
   CK(pool.alloc(&l, 1));
-  CK(launch_mlp_grad(params, x, y, B, (int)B, 0, 0, part, ploss, grad, l, s));
+  CK(launch_mlp_grad(params, x, y, B, (int)B, scratch, grad, l, s));
   if (loss) CK(cudaMemcpyAsync(loss, l, 4, cudaMemcpyDeviceToDevice, s));
   CK(cudaStreamSynchronize(s));
   return CNG_OK;

@@ -8,8 +8,16 @@
 // in the search kernel, label y = (t >= last hop at which the query's top-k list changed).
 // Inputs are standardised with the training set's per-feature mean and standard deviation.
 // Optimiser: Adam (beta 0.9 / 0.999, eps 1e-8); minibatch rows drawn with replacement by a
-// counter-based hash of (seed, step, slot).  Gradients: each CTA handles 128 samples and writes
-// its partial gradient; partials are summed in CTA order, so training is deterministic.
+// counter-based hash of (seed, step, slot).  Gradients: one partial per group of 128 samples, each
+// entry one sum over the group's samples in order; partials are summed in group order, so training
+// is deterministic.
+//
+// A step is three launches: activations and their gradients (32 samples a CTA, one sample per lane,
+// 8 outputs per warp), the groups' parameter gradients (eight CTAs a group), and the sum over the
+// groups with Adam's update.  Each sum keeps its order; what is parallel is the outputs.  Bound by the
+// dependent FMA chains, load latency and launches: a step of 4,096 samples took 90 us with one CTA of
+// 128 threads doing all of a group's work (32 CTAs in all), now 25 us (10.6 + 10 + 5); fitting on
+// 10,000 traces (384 steps) 35.8 -> 11.4 ms.
 #include "launch_count.h"
 #include "cng_internal.h"
 #include "device_common.cuh"
@@ -18,7 +26,11 @@
 
 namespace cng {
 
-constexpr int MT = 128;  // samples (threads) per CTA
+constexpr int MT = 128;  // samples per group (one partial gradient)
+constexpr int MA = 32;   // samples per CTA of the forward / backward kernel
+constexpr int MF = 256;  // its threads
+constexpr int MO = 64 / (MF / 32);  // outputs of a layer per warp
+constexpr int MG = 8;    // CTAs per group of the gradient kernel
 
 CNG_DEV uint64_t splitmix64(uint64_t x) {
   x += 0x9E3779B97F4A7C15ull;
@@ -144,122 +156,234 @@ __global__ void standardise_kernel(float* __restrict__ X, int64_t N, const float
 }
 
 // ---- forward + backward --------------------------------------------------------------------------
-// One thread per sample; rows = idx ? idx[i] : i.  Writes the CTA's partial gradient and loss.
-__global__ void __launch_bounds__(MT)
+// Activations and gradients of a batch, [samples rounded up to MT][..]: x 16, h1, h2, g1 (dL/da1) and
+// g2 (dL/da2) 64 each, dz and the loss 1 each.
+struct MlpActs {
+  float *x, *h1, *h2, *g1, *g2, *dz, *ls;
+};
+CNG_DEV void put4(float* p, const float* v) {
+  *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+static MlpActs acts_of(float* p, int B) {
+  const size_t n = (size_t)mlp_parts(B) * MT;
+  MlpActs a;
+  a.x = p;
+  a.h1 = a.x + n * 16;
+  a.h2 = a.h1 + n * 64;
+  a.g1 = a.h2 + n * 64;
+  a.g2 = a.g1 + n * 64;
+  a.dz = a.g2 + n * 64;
+  a.ls = a.dz + n;
+  return a;
+}
+
+// Rows drawn by hash of (seed, step, slot), or 0..B-1 (seed 0).  Lane = sample; warp w computes
+// outputs MO w .. + MO - 1 of each layer and keeps them in registers for the backward pass.
+__global__ void __launch_bounds__(MF)
 mlp_fwd_bwd_kernel(const float* __restrict__ P, const float* __restrict__ X, const float* __restrict__ Y,
-                   int64_t N, int B, uint64_t seed, int64_t step, float inv_scale,
-                   float* __restrict__ part, float* __restrict__ part_loss) {
-  extern __shared__ float sm[];
-  float* w = sm;                         // MLP_NPARAMS
-  float* xs = w + MLP_NPARAMS_PAD;       // [MT][16]
-  float* h1 = xs + MT * 16;              // [MT][65] (pad: conflict-free columns)
-  float* h2 = h1 + MT * 65;              // [MT][65]
-  float* g2 = h2 + MT * 65;              // [MT][65] dL/da2
-  float* g1 = g2 + MT * 65;              // [MT][65] dL/da1
-  __shared__ float dzs[MT];
-  __shared__ float ls[MT];
-  const int t = threadIdx.x;
-  for (int i = t; i < MLP_NPARAMS; i += MT) w[i] = P[i];
+                   int64_t N, int B, uint64_t seed, int64_t step, float inv_scale, MlpActs A) {
+  __shared__ __align__(16) float w[MLP_NPARAMS_PAD];
+  __shared__ float h1[MA * 65];  // [sample][65] (pad: conflict-free columns)
+  __shared__ float h2[MA * 65];  // later dL/da2
+  __shared__ float dzs[MA];
+  const int t = threadIdx.x, lane = t & 31, o0 = (t >> 5) * MO;
+  const int64_t s = (int64_t)blockIdx.x * MA + lane;
+  const bool live = s < B;
+  int64_t row = 0;
+  if (live) {
+    row = seed ? (int64_t)(splitmix64(seed ^ ((uint64_t)step * 0x100000001B3ull + (uint64_t)s)) %
+                           (uint64_t)N)
+               : s;
+  }
+  float x[16];
+#pragma unroll
+  for (int j = 0; j < 16; ++j) x[j] = live ? X[row * 16 + j] : 0.f;
+  const float y = live ? Y[row] : 0.f;
+  // every load of the weights in flight at once: a loop of dependent batches costs more than a layer
+#pragma unroll
+  for (int k = 0; k < (MLP_NPARAMS + MF - 1) / MF; ++k)
+    if (k * MF + t < MLP_NPARAMS) w[k * MF + t] = P[k * MF + t];
   const float* W1 = w;
   const float* b1 = W1 + 64 * 16;
   const float* W2 = b1 + 64;
   const float* b2 = W2 + 64 * 64;
   const float* w3 = b2 + 64;
   const float* b3 = w3 + 64;
-  const int s = blockIdx.x * MT + t;
-  const bool live = s < B;
-  int64_t row = 0;
-  if (live) {
-    row = seed ? (int64_t)(splitmix64(seed ^ ((uint64_t)step * 0x100000001B3ull + (uint64_t)s)) %
-                           (uint64_t)N)
-               : (int64_t)s;
-  }
-  for (int j = 0; j < 16; ++j) xs[t * 16 + j] = live ? X[row * 16 + j] : 0.f;
-  __syncthreads();
-  float z = b3[0];
-  for (int o = 0; o < 64; ++o) {
-    float a = b1[o];
+  if (o0 == 0) {
 #pragma unroll
-    for (int i = 0; i < 16; ++i) a = fmaf(W1[o * 16 + i], xs[t * 16 + i], a);
-    h1[t * 65 + o] = fmaxf(a, 0.f);
-  }
-  for (int o = 0; o < 64; ++o) {
-    float a = b2[o];
-    for (int i = 0; i < 64; ++i) a = fmaf(W2[o * 64 + i], h1[t * 65 + i], a);
-    float r = fmaxf(a, 0.f);
-    h2[t * 65 + o] = r;
-    z = fmaf(w3[o], r, z);
-  }
-  const float y = live ? Y[row] : 0.f;
-  const float sig = 1.f / (1.f + expf(-z));
-  const float dz = live ? (sig - y) * inv_scale : 0.f;
-  dzs[t] = dz;
-  ls[t] = live ? fmaxf(z, 0.f) - z * y + log1pf(expf(-fabsf(z))) : 0.f;
-  for (int o = 0; o < 64; ++o) g2[t * 65 + o] = h2[t * 65 + o] > 0.f ? dz * w3[o] : 0.f;
-  for (int i = 0; i < 64; ++i) {
-    float a = 0.f;
-    for (int o = 0; o < 64; ++o) a = fmaf(W2[o * 64 + i], g2[t * 65 + o], a);
-    g1[t * 65 + i] = h1[t * 65 + i] > 0.f ? a : 0.f;
+    for (int j = 0; j < 16; j += 4) put4(A.x + s * 16 + j, x + j);
   }
   __syncthreads();
-  // parameter gradients of this CTA's samples (fixed summation order over samples)
+  float r1[MO], a[MO];
+#pragma unroll
+  for (int k = 0; k < MO; ++k) {
+    r1[k] = b1[o0 + k];
+#pragma unroll
+    for (int i = 0; i < 16; i += 4) {
+      const float4 v = *reinterpret_cast<const float4*>(W1 + (o0 + k) * 16 + i);
+      r1[k] = fmaf(v.x, x[i], r1[k]);
+      r1[k] = fmaf(v.y, x[i + 1], r1[k]);
+      r1[k] = fmaf(v.z, x[i + 2], r1[k]);
+      r1[k] = fmaf(v.w, x[i + 3], r1[k]);
+    }
+    r1[k] = fmaxf(r1[k], 0.f);
+    h1[lane * 65 + o0 + k] = r1[k];
+    a[k] = b2[o0 + k];
+  }
+#pragma unroll
+  for (int k = 0; k < MO; k += 4) put4(A.h1 + s * 64 + o0 + k, r1 + k);
+  __syncthreads();
+#pragma unroll 4
+  for (int i = 0; i < 64; i += 4) {
+    const float* h = h1 + lane * 65 + i;
+    const float ha = h[0], hb = h[1], hc = h[2], hd = h[3];
+#pragma unroll
+    for (int k = 0; k < MO; ++k) {
+      const float4 v = *reinterpret_cast<const float4*>(W2 + (o0 + k) * 64 + i);
+      a[k] = fmaf(v.x, ha, a[k]);
+      a[k] = fmaf(v.y, hb, a[k]);
+      a[k] = fmaf(v.z, hc, a[k]);
+      a[k] = fmaf(v.w, hd, a[k]);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < MO; ++k) {
+    a[k] = fmaxf(a[k], 0.f);
+    h2[lane * 65 + o0 + k] = a[k];
+  }
+#pragma unroll
+  for (int k = 0; k < MO; k += 4) put4(A.h2 + s * 64 + o0 + k, a + k);
+  __syncthreads();
+  if (o0 == 0) {
+    float z = b3[0];
+#pragma unroll 16
+    for (int o = 0; o < 64; ++o) z = fmaf(w3[o], h2[lane * 65 + o], z);
+    const float sig = 1.f / (1.f + expf(-z));
+    const float dz = live ? (sig - y) * inv_scale : 0.f;
+    dzs[lane] = dz;
+    A.dz[s] = dz;
+    A.ls[s] = live ? fmaxf(z, 0.f) - z * y + log1pf(expf(-fabsf(z))) : 0.f;
+  }
+  __syncthreads();
+  const float dz = dzs[lane];
+#pragma unroll
+  for (int k = 0; k < MO; ++k) {
+    a[k] = a[k] > 0.f ? dz * w3[o0 + k] : 0.f;
+    h2[lane * 65 + o0 + k] = a[k];
+  }
+#pragma unroll
+  for (int k = 0; k < MO; k += 4) put4(A.g2 + s * 64 + o0 + k, a + k);
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < MO; ++k) a[k] = 0.f;
+#pragma unroll 8
+  for (int o = 0; o < 64; ++o) {
+    const float gv = h2[lane * 65 + o];
+#pragma unroll
+    for (int k = 0; k < MO; k += 4) {
+      const float4 v = *reinterpret_cast<const float4*>(W2 + o * 64 + o0 + k);
+      a[k] = fmaf(v.x, gv, a[k]);
+      a[k + 1] = fmaf(v.y, gv, a[k + 1]);
+      a[k + 2] = fmaf(v.z, gv, a[k + 2]);
+      a[k + 3] = fmaf(v.w, gv, a[k + 3]);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < MO; ++k) a[k] = r1[k] > 0.f ? a[k] : 0.f;
+#pragma unroll
+  for (int k = 0; k < MO; k += 4) put4(A.g1 + s * 64 + o0 + k, a + k);
+}
+
+// Parameter gradients of one group of MT samples (blockIdx.x), each entry a sum over the samples in
+// order.  blockIdx.y < 4: rows 16 y .. +15 of W2; 4: W1; 5: b1; 6: b2; 7: w3, b3 and the loss.  The
+// operands go to shared memory first: from global memory each step of the 128-step sums waited for a
+// load (49 us a launch for 32 groups, against 10).
+__global__ void __launch_bounds__(256) mlp_group_grad_kernel(MlpActs A, float* __restrict__ part,
+                                                             float* __restrict__ part_loss) {
+  __shared__ __align__(16) float wide[MT * 64];
+  __shared__ __align__(16) float slim[MT * 16];
+  const int t = threadIdx.x, y = blockIdx.y;
+  const int64_t s0 = (int64_t)blockIdx.x * MT;
   float* out = part + (size_t)blockIdx.x * MLP_NPARAMS;
-  for (int e = t; e < 64 * 16; e += MT) {  // W1[o][i]
-    int o = e >> 4, i = e & 15;
-    float a = 0.f;
-    for (int q = 0; q < MT; ++q) a = fmaf(g1[q * 65 + o], xs[q * 16 + i], a);
-    out[e] = a;
-  }
-  if (t < 64) {  // b1, b2, w3
-    float a = 0.f, c = 0.f, d = 0.f;
-    for (int q = 0; q < MT; ++q) {
-      a += g1[q * 65 + t];
-      c += g2[q * 65 + t];
-      d = fmaf(dzs[q], h2[q * 65 + t], d);
+  const float* src[4] = {A.g1, A.g1, A.g2, A.h2};
+  const float4* pw = reinterpret_cast<const float4*>((y < 4 ? A.h1 : src[y - 4]) + s0 * 64);
+#pragma unroll
+  for (int k = 0; k < MT * 16 / 256; ++k) reinterpret_cast<float4*>(wide)[k * 256 + t] = pw[k * 256 + t];
+  if (y < 5) {
+    // 16 floats a sample: the tile's columns of g2, or the sample's inputs
+    const float* ps = y < 4 ? A.g2 + s0 * 64 + 16 * y : A.x + s0 * 16;
+    const int ld = y < 4 ? 64 : 16;
+#pragma unroll
+    for (int k = 0; k < MT * 4 / 256; ++k) {
+      const int e = k * 256 + t;
+      reinterpret_cast<float4*>(slim)[e] = *reinterpret_cast<const float4*>(ps + (e >> 2) * ld + (e & 3) * 4);
     }
-    out[64 * 16 + t] = a;
-    out[64 * 16 + 64 + 64 * 64 + t] = c;
-    out[64 * 16 + 64 + 64 * 64 + 64 + t] = d;
+  } else if (y == 7) {
+    slim[t] = t < MT ? A.dz[s0 + t] : A.ls[s0 + t - MT];
   }
-  for (int e = t; e < 64 * 64; e += MT) {  // W2[o][i]
-    int o = e >> 6, i = e & 63;
-    float a = 0.f;
-    for (int q = 0; q < MT; ++q) a = fmaf(g2[q * 65 + o], h1[q * 65 + i], a);
-    out[64 * 16 + 64 + e] = a;
-  }
-  if (t == 0) {
-    float a = 0.f, l = 0.f;
+  __syncthreads();
+  if (y < 5) {  // thread = one of the 64 wide columns and 4 of the 16 slim ones
+    const int c = t & 63, f = (t >> 6) * 4;
+    float a[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 16
     for (int q = 0; q < MT; ++q) {
-      a += dzs[q];
-      l += ls[q];
+      const float v = wide[q * 64 + c];
+      const float4 g = *reinterpret_cast<const float4*>(slim + q * 16 + f);
+      a[0] = fmaf(g.x, v, a[0]);
+      a[1] = fmaf(g.y, v, a[1]);
+      a[2] = fmaf(g.z, v, a[2]);
+      a[3] = fmaf(g.w, v, a[3]);
     }
-    out[MLP_NPARAMS - 1] = a;
-    part_loss[blockIdx.x] = l;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      out[y < 4 ? 64 * 16 + 64 + (16 * y + f + k) * 64 + c : c * 16 + f + k] = a[k];
+  } else if (t < 64) {
+    float a = 0.f;
+    if (y < 7) {
+#pragma unroll 16
+      for (int q = 0; q < MT; ++q) a += wide[q * 64 + t];
+      out[y == 5 ? 64 * 16 + t : 64 * 16 + 64 + 64 * 64 + t] = a;
+    } else {
+#pragma unroll 16
+      for (int q = 0; q < MT; ++q) a = fmaf(slim[q], wide[q * 64 + t], a);
+      out[64 * 16 + 64 + 64 * 64 + 64 + t] = a;
+    }
+  } else if (y == 7 && (t == 64 || t == 96)) {
+    const float* v = t == 64 ? slim : slim + MT;
+    float a = 0.f;
+#pragma unroll 16
+    for (int q = 0; q < MT; ++q) a += v[q];
+    if (t == 64)
+      out[MLP_NPARAMS - 1] = a;
+    else
+      part_loss[blockIdx.x] = a;
   }
+}
+
+// The gradient from the groups' partials, summed in group order, and the mean loss.
+CNG_DEV float sum_parts(const float* __restrict__ part, int nparts, int p) {
+  float a = 0.f;
+#pragma unroll 32
+  for (int c = 0; c < nparts; ++c) a += part[(size_t)c * MLP_NPARAMS + p];
+  return a;
+}
+CNG_DEV void mean_loss(const float* __restrict__ part_loss, int nparts, float scale, float* loss) {
+  float l = 0.f;
+  for (int c = 0; c < nparts; ++c) l += part_loss[c];
+  *loss = l * scale;
 }
 
 __global__ void reduce_grad_kernel(const float* __restrict__ part, int nparts,
                                    const float* __restrict__ part_loss, float loss_scale,
                                    float* __restrict__ grad, float* __restrict__ loss) {
   int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p < MLP_NPARAMS) {
-    float a = 0.f;
-    for (int c = 0; c < nparts; ++c) a += part[(size_t)c * MLP_NPARAMS + p];
-    grad[p] = a;
-  }
-  if (p == 0 && loss) {
-    float l = 0.f;
-    for (int c = 0; c < nparts; ++c) l += part_loss[c];
-    *loss = l * loss_scale;
-  }
+  if (p < MLP_NPARAMS) grad[p] = sum_parts(part, nparts, p);
+  if (p == 0 && loss) mean_loss(part_loss, nparts, loss_scale, loss);
 }
 
-__global__ void adam_kernel(float* __restrict__ P, float* __restrict__ m, float* __restrict__ v,
-                            const float* __restrict__ g, int64_t t, float lr) {
-  int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= MLP_NPARAMS) return;
+CNG_DEV void adam_update(float* __restrict__ P, float* __restrict__ m, float* __restrict__ v, int p,
+                         float gi, int64_t t, float lr) {
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-  float gi = g[p];
   float mi = b1 * m[p] + (1.f - b1) * gi;
   float vi = b2 * v[p] + (1.f - b2) * gi * gi;
   m[p] = mi;
@@ -267,6 +391,24 @@ __global__ void adam_kernel(float* __restrict__ P, float* __restrict__ m, float*
   float mh = mi / (1.f - powf(b1, (float)t));
   float vh = vi / (1.f - powf(b2, (float)t));
   P[p] -= lr * mh / (sqrtf(vh) + eps);
+}
+
+__global__ void adam_kernel(float* __restrict__ P, float* __restrict__ m, float* __restrict__ v,
+                            const float* __restrict__ g, int64_t t, float lr) {
+  int p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= MLP_NPARAMS) return;
+  adam_update(P, m, v, p, g[p], t, lr);
+}
+
+// The last launch of a training step: gradient, loss (if wanted) and Adam's update.
+__global__ void reduce_adam_kernel(const float* __restrict__ part, int nparts,
+                                   const float* __restrict__ part_loss, float loss_scale,
+                                   float* __restrict__ loss, float* __restrict__ P, float* __restrict__ m,
+                                   float* __restrict__ v, int64_t t, float lr) {
+  int p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p == 0 && loss) mean_loss(part_loss, nparts, loss_scale, loss);
+  if (p >= MLP_NPARAMS) return;
+  adam_update(P, m, v, p, sum_parts(part, nparts, p), t, lr);
 }
 
 // Kaiming-uniform weights, zero biases, from the counter-based generator.
@@ -316,21 +458,47 @@ __global__ void pack_model_kernel(const float* __restrict__ P, const float* __re
 }
 
 // ---- host-side launchers ---------------------------------------------------------------------------
-size_t mlp_fwd_bwd_smem() { return (size_t)(MLP_NPARAMS_PAD + MT * 16 + 4 * MT * 65) * sizeof(float); }
 int mlp_parts(int B) { return (B + MT - 1) / MT; }
+size_t mlp_scratch_floats(int B) {
+  const size_t n = (size_t)mlp_parts(B) * MT;
+  return (size_t)mlp_parts(B) * (MLP_NPARAMS + 1) + 4 + n * (16 + 4 * 64 + 2);
+}
+
+// scratch: the groups' losses, their partial gradients, the activations (16-byte aligned)
+static cudaError_t launch_partials(const float* P, const float* X, const float* Y, int64_t N, int B,
+                                   uint64_t seed, int64_t step, float* scratch, float** part,
+                                   float** part_loss, cudaStream_t s) {
+  const int parts = mlp_parts(B);
+  *part_loss = scratch;
+  *part = scratch + parts;
+  const MlpActs A = acts_of(scratch + ((size_t)parts * (MLP_NPARAMS + 1) + 3) / 4 * 4, B);
+  count_launch();
+  mlp_fwd_bwd_kernel<<<parts * (MT / MA), MF, 0, s>>>(P, X, Y, N, B, seed, step, 1.f / (float)B, A);
+  count_launch();
+  mlp_group_grad_kernel<<<dim3(parts, MG), 256, 0, s>>>(A, *part, *part_loss);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_mlp_grad(const float* P, const float* X, const float* Y, int64_t N, int B,
-                            uint64_t seed, int64_t step, float* part, float* part_loss, float* grad,
-                            float* loss, cudaStream_t s) {
-  const size_t sh = mlp_fwd_bwd_smem();
-  cudaError_t e = cudaFuncSetAttribute(mlp_fwd_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
+                            float* scratch, float* grad, float* loss, cudaStream_t s) {
+  float *part, *part_loss;
+  cudaError_t e = launch_partials(P, X, Y, N, B, 0, 0, scratch, &part, &part_loss, s);
   if (e != cudaSuccess) return e;
-  const int parts = mlp_parts(B);
   count_launch();
-  mlp_fwd_bwd_kernel<<<parts, MT, sh, s>>>(P, X, Y, N, B, seed, step, 1.f / (float)B, part, part_loss);
+  reduce_grad_kernel<<<(MLP_NPARAMS + 255) / 256, 256, 0, s>>>(part, mlp_parts(B), part_loss,
+                                                               1.f / (float)B, grad, loss);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_mlp_step(float* P, const float* X, const float* Y, int64_t N, int B, uint64_t seed,
+                            int64_t t, float lr, float* m, float* v, float* scratch, float* loss,
+                            cudaStream_t s) {
+  float *part, *part_loss;
+  cudaError_t e = launch_partials(P, X, Y, N, B, seed, t, scratch, &part, &part_loss, s);
+  if (e != cudaSuccess) return e;
   count_launch();
-  reduce_grad_kernel<<<(MLP_NPARAMS + 255) / 256, 256, 0, s>>>(part, parts, part_loss, 1.f / (float)B,
-                                                               grad, loss);
+  reduce_adam_kernel<<<(MLP_NPARAMS + 127) / 128, 128, 0, s>>>(part, mlp_parts(B), part_loss,
+                                                               1.f / (float)B, loss, P, m, v, t, lr);
   return cudaGetLastError();
 }
 

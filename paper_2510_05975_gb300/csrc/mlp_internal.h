@@ -10,13 +10,16 @@ namespace cng {
 constexpr int MLP_NPARAMS = 64 * 16 + 64 + 64 * 64 + 64 + 64 + 1;  // 5313
 constexpr int MLP_NPARAMS_PAD = 5316;
 
-size_t mlp_fwd_bwd_smem();
 int mlp_parts(int B);
-// Gradient of the mean loss over B rows (rows drawn by hash of (seed, step) when seed != 0,
-// else rows 0..B-1).  part: mlp_parts(B) * MLP_NPARAMS floats; part_loss: mlp_parts(B).
+size_t mlp_scratch_floats(int B);  // floats of scratch (16-byte aligned) for a batch of B rows
+// Gradient of the mean loss over rows 0..B-1.
 cudaError_t launch_mlp_grad(const float* P, const float* X, const float* Y, int64_t N, int B,
-                            uint64_t seed, int64_t step, float* part, float* part_loss, float* grad,
-                            float* loss, cudaStream_t s);
+                            float* scratch, float* grad, float* loss, cudaStream_t s);
+// One training step: B rows drawn by hash of (seed, t), their gradient and Adam's update; *loss (if
+// not null) receives the mean loss.
+cudaError_t launch_mlp_step(float* P, const float* X, const float* Y, int64_t N, int B, uint64_t seed,
+                            int64_t t, float lr, float* m, float* v, float* scratch, float* loss,
+                            cudaStream_t s);
 cudaError_t launch_adam(float* P, float* m, float* v, const float* g, int64_t t, float lr,
                         cudaStream_t s);
 cudaError_t launch_mlp_init(float* P, uint64_t seed, cudaStream_t s);
