@@ -314,7 +314,6 @@ static cng_status run_knn(const KnnInputs& in, int32_t* out_ids, float* out_dist
     ta.ids = sids;
     ta.thr = sthr;
     ta.status = &ctr->status;
-    ta.rowbuf_words = screen_tc_rowbuf_words(in.m, in.n, in.Lp);
     ta.perm = in.perm;
     ta.wave_start = in.wave_start;
     ta.variant = in.variant;
@@ -322,6 +321,7 @@ static cng_status run_knn(const KnnInputs& in, int32_t* out_ids, float* out_dist
     ta.col_perm = in.col_perm;
     ta.col_pos = in.col_pos;
     for (int i = 0; i < RES_PARTS; ++i) ta.part_count[i] = in.part_count[i];
+    ta.rowbuf_words = screen_tc_rowbuf_words(ta);
     CK(pool.alloc(&ta.rowbuf, ta.rowbuf_words));
     std::string msg;
     if (in.variant < 0) {  // a first use of this shape times the variants (outside the timing)
@@ -1719,8 +1719,6 @@ static cng_status tc_scores(const float* rows, int64_t m, const float* cols, int
   ta.Lp = 32;
   ta.self_excl = 0;
   ta.status = status;
-  ta.rowbuf_words = screen_tc_rowbuf_words(m, n, 32);
-  CK(pool.alloc(&ta.rowbuf, ta.rowbuf_words));
   if (res_shape(d, bits_to_float(pc.st.nbmax_bits), &ta.res)) {
     char *ri, *ci;
     CK(pool.alloc(&ri, res_image_bytes(ta.res, m)));
@@ -1730,6 +1728,8 @@ static cng_status tc_scores(const float* rows, int64_t m, const float* cols, int
     ta.A = ri;
     ta.B = ci;
   }
+  ta.rowbuf_words = screen_tc_rowbuf_words(ta);
+  CK(pool.alloc(&ta.rowbuf, ta.rowbuf_words));
   std::string msg;
   cudaError_t e = launch_screen_tc_dump(ta, scores, s, &msg);
   if (e != cudaSuccess) return fail(CNG_E_CUDA, "tensor-core screen: " + msg + cudaGetErrorString(e));

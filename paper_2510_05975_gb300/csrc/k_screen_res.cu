@@ -35,7 +35,7 @@
 // which the tensor pipe, which queues only a few MMAs, would idle (one issuer for all: 1,680
 // cycles per 256 x 80 tile; two: 1,260; four: 840, against 890 for the 18 MMAs alone at 49 each).
 //
-// Bound: without hits the tensor pipe (1,900 TFLOP/s of kt-wide products); the appends add ~40%.
+// Bound: without hits the tensor pipe (1,900 TFLOP/s of 2 m n d at d = 128); the appends add ~40%.
 // 1M x 128, L' = 160, self: 202 ms, 1,265 TFLOP/s of 2 n^2 d (0.74 of the measured sustained bf16
 // rate), against 402 ms for the kernel before (rows in shared memory, one issuer, thresholds that
 // fall during the sweep); 1M x 96, L' = 192: 431 -> 189 ms.
@@ -75,6 +75,10 @@ struct ResParams {
   int npart;                     // sweep parts: tiles [.., part_end[i]) kept to rank part_rank[i]
   int part_end[RES_PARTS];
   int part_rank[RES_PARTS];
+  int nsplit, pre;               // column split: units = row blocks x nsplit, whole tiles up to pre
+  uint64_t* mlist;               // [nsplit][m][Lp] a unit's keys (nsplit > 1), their number and the
+  int32_t* mcnt;                 // [nsplit][m]     unit's threshold key
+  uint32_t* mthr;
   uint16_t aux[RES_AUX];         // the row constants -c_i as operand bits
   const int32_t* row_perm;       // point id of a row position (null: the position)
   const int32_t* col_perm;       // point id of a column position (null: the position)
@@ -226,6 +230,23 @@ CNG_DEV uint32_t warp_cut(uint64_t* buf, int cnt, int need, int slack, int lane,
   return __reduce_max_sync(FULL, top);
 }
 
+// A unit of work is a row block and a split of the columns: the tiles up to P.pre (sample parts, for
+// the thresholds), then every nsplit-th of the rest from the split's own on.
+struct ResUnit {
+  int64_t rb;
+  int split, ntiles;
+};
+CNG_DEV ResUnit res_unit(const ResParams& P, int64_t u, int64_t nrb) {
+  ResUnit r;
+  r.split = (int)(u / nrb);
+  r.rb = u - r.split * nrb;
+  r.ntiles = P.pre + (P.ntiles - P.pre - r.split + P.nsplit - 1) / P.nsplit;
+  return r;
+}
+CNG_DEV int res_tile(const ResParams& P, const ResUnit& r, int t) {
+  return t < P.pre ? t : P.pre + r.split + (t - P.pre) * P.nsplit;
+}
+
 // Appends one row's (lane's) columns of the chunk [c0, c0 + 16) whose accumulators beat its
 // threshold; mx is the chunk's maximum, so a single hit needs no search for its value (a second one
 // in the same chunk is rare after the first tiles and picks its value by a select chain).
@@ -268,6 +289,7 @@ __global__ void __launch_bounds__(rs_threads(NBUF), 1) screen_res_kernel(const _
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int64_t nrb = (P.m + RS_BM - 1) / RS_BM;
+  const int64_t nunits = nrb * P.nsplit;
 
   if (tid == 0) {
     for (int i = 0; i < P.nst; ++i) {
@@ -300,13 +322,14 @@ __global__ void __launch_bounds__(rs_threads(NBUF), 1) screen_res_kernel(const _
       int s = 0;
       uint32_t ph = 0;
       bool ok = true;
-      for (int64_t rb = blockIdx.x; rb < nrb && ok; rb += gridDim.x) {
-        for (int t = 0; t < P.ntiles; ++t, ++it) {
+      for (int64_t u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
+        const ResUnit un = res_unit(P, u, nrb);
+        for (int t = 0; t < un.ntiles; ++t, ++it) {
           wave_checkpoint(P.sync, P.sync_d, TC_SYNC_COLS / BN, it, nrb, P.ntiles);
           ok = mbar_wait(&b_empty[s], ph ^ 1, abort_flag, P.status);
           if (!ok) break;
           mbar_expect_tx(&b_full[s], (uint32_t)stage_bytes);
-          bulk_load(sB + s * stage_bytes, P.B + (size_t)t * stage_bytes, (uint32_t)stage_bytes, &b_full[s]);
+          bulk_load(sB + s * stage_bytes, P.B + (size_t)res_tile(P, un, t) * stage_bytes, (uint32_t)stage_bytes, &b_full[s]);
           if (++s == P.nst) {
             s = 0;
             ph ^= 1u;
@@ -336,11 +359,12 @@ __global__ void __launch_bounds__(rs_threads(NBUF), 1) screen_res_kernel(const _
       uint64_t* const tf = &t_full[half * NBUF + b];
       uint64_t* const te = &t_empty[half * NBUF + b];
       uint64_t* const fn = &fin[half * NBUF + b];
-      for (int64_t rb = blockIdx.x; rb < nrb && ok; rb += gridDim.x, ++j) {
+      for (int64_t u = blockIdx.x; u < nunits && ok; u += gridDim.x, ++j) {
+        const int ntiles = res_unit(P, u, nrb).ntiles;
         ok = mbar_wait(&a_full[half], j & 1, abort_flag, P.status);
         if (!ok) break;
         tc_fence_after();
-        for (int t = 0; t < P.ntiles; ++t) {
+        for (int t = 0; t < ntiles; ++t) {
           if (turn == b) {
             ok = mbar_wait(&b_full[s], sph, abort_flag, P.status);
             if (!ok) break;
@@ -396,8 +420,9 @@ __global__ void __launch_bounds__(rs_threads(NBUF), 1) screen_res_kernel(const _
     int b = 0;
     uint32_t bph = 0;
     bool ok = true;
-    for (int64_t rb = blockIdx.x; rb < nrb && ok; rb += gridDim.x) {
-      const int64_t row = rb * RS_BM + rloc;
+    for (int64_t u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
+      const ResUnit un = res_unit(P, u, nrb);
+      const int64_t row = un.rb * RS_BM + rloc;
       const bool live = row < P.m;
       {
         // the row's operand into TMEM: every MMA of the previous block is complete (this warp
@@ -432,7 +457,7 @@ __global__ void __launch_bounds__(rs_threads(NBUF), 1) screen_res_kernel(const _
       const uint32_t self = P.self_excl && live ? (uint32_t)P.col_pos[P.row_perm[row]] : ~0u;
       int t = 0;
       for (int part = 0; part < P.npart && ok; ++part) {
-        const int tend = P.part_end[part];
+        const int tend = part + 1 == P.npart ? un.ntiles : P.part_end[part];
         const int rank = P.part_rank[part];
         for (; t < tend; ++t) {
           ok = mbar_wait_warp(&tf[b], bph, abort_flag, P.status);
@@ -455,6 +480,7 @@ __global__ void __launch_bounds__(rs_threads(NBUF), 1) screen_res_kernel(const _
               for (int j = 0; j < BN; ++j)
                 if (c0 + j < P.n) dump[row * P.n + c0 + j] = -2.f * __uint_as_float(r[j]);
           } else {
+            const int tile = res_tile(P, un, t);
             float m[BN / RS_C];
 #pragma unroll
             for (int c = 0; c < BN / RS_C; ++c) m[c] = max16<BN>(r, c * RS_C);
@@ -465,7 +491,7 @@ __global__ void __launch_bounds__(rs_threads(NBUF), 1) screen_res_kernel(const _
 #pragma unroll
               for (int c = 0; c < BN / RS_C; ++c)
                 if (m[c] > thr)
-                  append_chunk<BN>(r, c * RS_C, m[c], (uint32_t)(t * BN + c * RS_C), (uint32_t)P.n, self,
+                  append_chunk<BN>(r, c * RS_C, m[c], (uint32_t)(tile * BN + c * RS_C), (uint32_t)P.n, self,
                                    thr, rbuf, cnt);
               // cut every list that could overflow on the next tile
               unsigned full = __ballot_sync(FULL, cnt > P.cap - BN);
@@ -481,6 +507,7 @@ __global__ void __launch_bounds__(rs_threads(NBUF), 1) screen_res_kernel(const _
         // end of a sample part: every list down to the part's rank
         __syncwarp();
         for (int l = 0; l < 32; ++l) cut(l, rank, 0);
+        if (part + 2 == P.npart && un.split > 0) cnt = 0;  // split 0 lists the sample's columns
       }
       if (!ok || DUMP) continue;
       // the Lp smallest of each list, ids and threshold key
@@ -493,6 +520,15 @@ __global__ void __launch_bounds__(rs_threads(NBUF), 1) screen_res_kernel(const _
         uint64_t* buf_l = wbuf + (size_t)l * P.cap;
         uint32_t key = isinf(t_l) ? 0xffffffffu : fkey(-2.f * t_l);
         if (c_l > P.Lp) key = warp_cut<CPL>(buf_l, c_l, P.Lp, 0, lane, &c_l);
+        if (P.nsplit > 1) {
+          const int64_t at = un.split * P.m + row_l;
+          for (int i = lane; i < c_l; i += 32) P.mlist[at * P.Lp + i] = buf_l[i];
+          if (lane == 0) {
+            P.mcnt[at] = c_l;
+            P.mthr[at] = key;
+          }
+          continue;
+        }
         const int64_t orow = P.row_perm ? P.row_perm[row_l] : row_l;
         for (int i = lane; i < P.Lp; i += 32) {
           int32_t id = -1;
@@ -513,6 +549,45 @@ __global__ void __launch_bounds__(rs_threads(NBUF), 1) screen_res_kernel(const _
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
   }
+}
+
+// The Lp smallest of a row's keys over its splits, one warp per row.  A column that is not listed lies
+// at or above the smallest of the splits' thresholds and of the cuts made here.
+constexpr int RS_MCAP = 24 * 32;
+__global__ void __launch_bounds__(256) screen_merge_kernel(const __grid_constant__ ResParams P) {
+  __shared__ uint64_t bufs[8][RS_MCAP];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t row = (int64_t)blockIdx.x * 8 + warp;
+  if (row >= P.m) return;
+  uint64_t* buf = bufs[warp];
+  uint32_t thr = 0xffffffffu;
+  int cnt = 0;
+  // lists are complete only if the screen's waits were: otherwise (the call fails) empty lists
+  const int nsplit = *reinterpret_cast<volatile uint32_t*>(P.status) ? 0 : P.nsplit;
+  for (int sp = 0; sp < nsplit; ++sp) {
+    const int64_t at = sp * P.m + row;
+    const int c = P.mcnt[at];
+    thr = min(thr, P.mthr[at]);
+    for (int i = 0; i < c;) {
+      const int take = min(c - i, RS_MCAP - cnt);
+      for (int j = lane; j < take; j += 32) buf[cnt + j] = P.mlist[at * P.Lp + i + j];
+      __syncwarp();
+      i += take;
+      cnt += take;
+      if (cnt == RS_MCAP) thr = min(thr, warp_cut<24>(buf, cnt, P.Lp, 0, lane, &cnt));
+    }
+  }
+  if (cnt > P.Lp) thr = min(thr, warp_cut<24>(buf, cnt, P.Lp, 0, lane, &cnt));
+  const int64_t orow = P.row_perm ? P.row_perm[row] : row;
+  for (int i = lane; i < P.Lp; i += 32) {
+    int32_t id = -1;
+    if (i < cnt) {
+      id = key_id(buf[i]);
+      if (P.col_perm) id = P.col_perm[id];
+    }
+    P.ids[orow * P.Lp + i] = id;
+  }
+  if (lane == 0) P.thr[orow] = thr;
 }
 
 // ---- operand images ----------------------------------------------------------------------------
@@ -665,6 +740,94 @@ static void schedule(const TcScreenArgs& a, int bn, int ntiles, ResParams* p) {
   p->part_rank[p->npart++] = a.Lp;
 }
 
+// List capacity: the last part appends about 1.3 Lp to the sample's rank; one size up if asked.
+static int list_cap(int Lp, int step) {
+  static const int caps[] = {12, 16, 20, 24};
+  int ci = 0;
+  while (ci < 3 && caps[ci] * 32 < 2 * Lp + 128) ++ci;
+  return caps[std::min(3, ci + step)] * 32;
+}
+
+// Column split for launches whose row blocks leave SMs idle (fewer than 4 per SM and no multiple of
+// them): the split and the sample parts swept whole by each unit that minimise
+//   waves x (unit overhead + sample tiles + other tiles / splits + hits),
+// in tiles of ~850 cycles; a hit per row costs ~6 tiles (32 rows append in turn), a unit's operand
+// load and final lists ~40, merging the splits' lists ~60.  10,000 rows against 1M x 128 (40 row
+// blocks): 3 splits with the 1/16 sample, 8.0 -> 4.2 ms.  With many row blocks nothing is gained: the
+// sample would be swept once per split.
+static void split_columns(int64_t nrb, int bn, int64_t n, int Lp, int cap, ResParams* p) {
+  p->nsplit = 1;
+  p->pre = 0;
+  const int64_t sms = num_sms();
+  if (nrb >= 4 * sms) return;
+  const double hit = 6.0, unit = 40.0, merge = 60.0;
+  auto fill = [&](double cols, int rank) {  // appends of a list that starts empty: rows append at once
+    return 0.4 * (cols <= cap ? cols : cap + rank * std::log(cols / cap));
+  };
+  // appends per row up to the end of each part
+  double upto[RES_PARTS], frac[RES_PARTS];
+  for (int i = 0; i < p->npart; ++i) {
+    frac[i] = std::min(1.0, (double)p->part_end[i] * bn / (double)n);
+    upto[i] = i == 0 ? fill(frac[0] * (double)n, p->part_rank[0])
+                     : upto[i - 1] + p->part_rank[i - 1] * (frac[i] / frac[i - 1] - 1.0);
+  }
+  double best = (double)((nrb + sms - 1) / sms) * (unit + p->ntiles + hit * upto[p->npart - 1]);
+  int best_k = -2;
+  for (int k = -1; k + 1 < p->npart; ++k) {
+    const int pre = k < 0 ? 0 : p->part_end[k];
+    for (int64_t sp = 2; sp * nrb <= 4 * sms && sp <= sms && sp * 4 <= p->ntiles - pre; ++sp) {
+      const double h = k < 0 ? fill((double)n / (double)sp, Lp)
+                             : upto[k] + p->part_rank[k] * (1.0 / frac[k] - 1.0) / (double)sp;
+      const double c = merge + (double)((nrb * sp + sms - 1) / sms) *
+                                   (unit + pre + (double)(p->ntiles - pre) / (double)sp + hit * h);
+      if (c < best) {
+        best = c;
+        best_k = k;
+        p->nsplit = (int)sp;
+        p->pre = pre;
+      }
+    }
+  }
+  if (p->nsplit == 1) return;
+  p->npart = best_k + 2;  // the parts swept whole, then the unit's share of the rest
+  p->part_end[best_k + 1] = p->ntiles;
+  p->part_rank[best_k + 1] = Lp;
+}
+
+// Row buffers, then the checkpoint counters (one split) or the splits' lists, in 8-byte words.
+struct ResScratch {
+  int grid;
+  size_t buf, sync, total;
+};
+static ResScratch res_scratch(int64_t m, int bn, const ResParams& p) {
+  const int64_t nrb = (m + RS_BM - 1) / RS_BM;
+  ResScratch r;
+  r.grid = (int)std::min<int64_t>(nrb * p.nsplit, num_sms());
+  r.buf = (size_t)r.grid * RS_BM * p.cap;
+  const int64_t waves = (nrb + r.grid - 1) / r.grid;
+  r.sync = p.nsplit > 1 ? 0 : (size_t)((waves * p.ntiles / (TC_SYNC_COLS / bn) + 3) / 2);
+  r.total = r.buf + r.sync + (p.nsplit > 1 ? (size_t)m * p.nsplit * (p.Lp + 1) : 0);
+  return r;
+}
+
+static void plan_res(const TcScreenArgs& a, int cap_step, bool split, ResParams* p) {
+  const int bn = a.res.bn;
+  p->ntiles = (int)((a.n + bn - 1) / bn);
+  p->Lp = a.Lp;
+  p->cap = list_cap(a.Lp, cap_step);
+  schedule(a, bn, p->ntiles, p);
+  p->nsplit = 1;
+  p->pre = 0;
+  if (split) split_columns((a.m + RS_BM - 1) / RS_BM, bn, a.n, a.Lp, p->cap, p);
+}
+
+size_t screen_res_rowbuf_words(const TcScreenArgs& a, int cap_step) {
+  ResParams p{}, whole{};  // the test aid that dumps scores does not split
+  plan_res(a, cap_step, true, &p);
+  plan_res(a, cap_step, false, &whole);
+  return std::max(res_scratch(a.m, a.res.bn, p).total, res_scratch(a.m, a.res.bn, whole).total);
+}
+
 template <int BN, int NBUF, int CPL, bool DUMP>
 static cudaError_t launch_res_t(const ResParams& p, size_t smem, int grid, cudaStream_t s, float* dump) {
   cudaError_t e = cudaFuncSetAttribute(screen_res_kernel<BN, NBUF, CPL, DUMP>,
@@ -713,21 +876,14 @@ cudaError_t launch_screen_res(const TcScreenArgs& a, const TcVariant& v, int var
   p.n = a.n;
   p.kt = kt;
   p.d = a.res.d;
-  p.ntiles = (int)((a.n + bn - 1) / bn);
+  plan_res(a, v.cap_step, a.split && !dump, &p);
   const int stage_bytes = bn * kt * 2;
   const int fixed = (2 * RS_MAXST + 14) * 8 + 16;
   p.nst = std::min(RS_MAXST, (226 * 1024 - fixed) / stage_bytes) - v.stages_less;
-  p.Lp = a.Lp;
-  // list capacity: the last part appends about 1.3 Lp to the sample's rank; one size up if asked
-  static const int caps[] = {12, 16, 20, 24};
-  int ci = 0;
-  while (ci < 3 && caps[ci] * 32 < 2 * a.Lp + 128) ++ci;
-  ci = std::min(3, ci + v.cap_step);
-  if (caps[ci] * 32 < a.Lp + 128) {
+  if (p.cap < a.Lp + 128) {
     if (msg) *msg = "screened list too long; ";
     return cudaErrorInvalidValue;
   }
-  p.cap = caps[ci] * 32;
   p.sync_d = v.sync_d;
   if (shape) *shape = TcShape{variant, p.nst, p.cap, p.sync_d};
   p.self_excl = a.self_excl;
@@ -742,7 +898,6 @@ cudaError_t launch_screen_res(const TcScreenArgs& a, const TcVariant& v, int var
   p.A = static_cast<const unsigned char*>(a.A);
   p.B = static_cast<const unsigned char*>(a.B);
   p.row0 = a.row_off;
-  schedule(a, bn, p.ntiles, &p);
   const AuxScale ax = aux_scales(a.fp16 != 0);
   for (int i = 0; i < RES_AUX; ++i) {
     if (a.fp16) {
@@ -761,26 +916,31 @@ cudaError_t launch_screen_res(const TcScreenArgs& a, const TcVariant& v, int var
   p.ids = a.ids;
   p.thr = a.thr;
   p.status = a.status;
-  const int64_t nrb = (a.m + RS_BM - 1) / RS_BM;
-  const int grid = (int)std::min<int64_t>(nrb, num_sms());
+  const ResScratch sc = res_scratch(a.m, bn, p);
   // at least ~116 KB so that a single CTA (and its 512 TMEM columns) fits per SM
   const size_t smem = std::max<size_t>((size_t)fixed + (size_t)p.nst * stage_bytes, 116 * 1024);
-  const size_t buf_words = (size_t)grid * RS_BM * p.cap;
-  const int64_t waves = (nrb + grid - 1) / grid;
-  const size_t sync_words = (size_t)((waves * p.ntiles / (TC_SYNC_COLS / bn) + 3) / 2);
-  if (!a.rowbuf || a.rowbuf_words < buf_words + (dump ? 0 : sync_words)) {
+  if (!a.rowbuf || a.rowbuf_words < sc.total) {
     if (msg) *msg = "row buffer missing or too small; ";
     return cudaErrorInvalidValue;
   }
   p.rowbuf = a.rowbuf;
-  if (!dump) {  // checkpoint counters after the row buffers, zeroed on the stream
-    p.sync = reinterpret_cast<uint32_t*>(a.rowbuf + buf_words);
-    cudaError_t ze = cudaMemsetAsync(p.sync, 0, sync_words * 8, s);
+  if (p.nsplit > 1) {
+    p.mlist = a.rowbuf + sc.buf;
+    p.mcnt = reinterpret_cast<int32_t*>(p.mlist + (size_t)a.m * p.nsplit * p.Lp);
+    p.mthr = reinterpret_cast<uint32_t*>(p.mcnt + (size_t)a.m * p.nsplit);
+  } else if (!dump) {  // checkpoint counters after the row buffers, zeroed on the stream
+    p.sync = reinterpret_cast<uint32_t*>(a.rowbuf + sc.buf);
+    cudaError_t ze = cudaMemsetAsync(p.sync, 0, sc.sync * 8, s);
     if (ze != cudaSuccess) return ze;
   }
-  if (bn == 96) return launch_res_bn<96, 2>(p.cap / 32, p, smem, grid, s, dump);
-  if (bn == 80) return launch_res_bn<80, 2>(p.cap / 32, p, smem, grid, s, dump);
-  return launch_res_bn<64, 2>(p.cap / 32, p, smem, grid, s, dump);
+  const int cpl = p.cap / 32;
+  cudaError_t e = bn == 96   ? launch_res_bn<96, 2>(cpl, p, smem, sc.grid, s, dump)
+                  : bn == 80 ? launch_res_bn<80, 2>(cpl, p, smem, sc.grid, s, dump)
+                             : launch_res_bn<64, 2>(cpl, p, smem, sc.grid, s, dump);
+  if (e != cudaSuccess || p.nsplit == 1) return e;
+  count_launch();
+  screen_merge_kernel<<<(unsigned)((a.m + 7) / 8), 256, 0, s>>>(p);
+  return cudaGetLastError();
 }
 
 }  // namespace cng

@@ -797,6 +797,11 @@ constexpr int TC_NVARIANTS = (int)(sizeof(TC_VARIANTS) / sizeof(TC_VARIANTS[0]))
 
 int screen_tc_variants() { return TC_NVARIANTS; }
 
+// Rows of the autotuner's sample: two waves of row blocks.
+static int64_t tune_sample(int64_t m) {
+  return 2 * TC_BM * std::min<int64_t>((m + TC_BM - 1) / TC_BM, num_sms());
+}
+
 static cudaError_t launch_impl(const TcScreenArgs& a, cudaStream_t s, std::string* msg, float* dump,
                                int variant, TcShape* shape) {
   if (variant < 0 || variant >= TC_NVARIANTS) {
@@ -882,11 +887,17 @@ static cudaError_t launch_impl(const TcScreenArgs& a, cudaStream_t s, std::strin
   return e;
 }
 
-size_t screen_tc_rowbuf_words(int64_t m, int64_t n, int Lp) {
+// The autotuner times variants on samples of at most m rows, one of them with larger lists.
+size_t screen_tc_rowbuf_words(const TcScreenArgs& a) {
+  if (a.res.kt > 0) {
+    const bool tuned = a.variant < 0 && a.m >= 4 * tune_sample(a.m);
+    const int step = a.variant >= 0 && a.variant < TC_NVARIANTS ? TC_VARIANTS[a.variant].cap_step : (tuned ? 1 : 0);
+    return screen_res_rowbuf_words(a, step);
+  }
   const int cpl = 24;  // the largest capacity launch_impl may choose
-  const int64_t nrb = (m + TC_BM - 1) / TC_BM;
+  const int64_t nrb = (a.m + TC_BM - 1) / TC_BM;
   const int grid = (int)std::min<int64_t>(nrb, num_sms());
-  return (size_t)grid * TC_BM * cpl * 32 + sync_counter_words(m, n, grid);
+  return (size_t)grid * TC_BM * cpl * 32 + sync_counter_words(a.m, a.n, grid);
 }
 
 // ---- autotuner -----------------------------------------------------------------------------------
@@ -910,8 +921,7 @@ static int tune_key_nlog(int64_t n) {
 
 static cudaError_t tune_variant(const TcScreenArgs& a, cudaStream_t s, std::string* msg, int* chosen) {
   *chosen = 0;
-  const int64_t grid = std::min<int64_t>((a.m + TC_BM - 1) / TC_BM, num_sms());
-  const int64_t sample = 2 * grid * TC_BM;
+  const int64_t sample = tune_sample(a.m);
   if (a.m < 4 * sample) return cudaSuccess;  // small problems: the default variant
   int dev = 0;
   cudaGetDevice(&dev);
@@ -942,6 +952,7 @@ static cudaError_t tune_variant(const TcScreenArgs& a, cudaStream_t s, std::stri
     t.m = sample;
     t.self_excl = 0;
     t.perm = nullptr;
+    t.split = 0;
     t.ids = ids;
     t.thr = thr;
     t.status = st;

@@ -43,7 +43,7 @@ struct TcScreenArgs {
   int32_t* ids;       // [m][Lp] screened ids (unordered), -1 padded
   uint32_t* thr;      // [m] ordered key of the largest kept score (0xffffffff: all kept)
   uint32_t* status;
-  uint64_t* rowbuf;     // scratch: screen_tc_rowbuf_words(m, n, Lp) words
+  uint64_t* rowbuf;     // scratch: screen_tc_rowbuf_words() words
   size_t rowbuf_words;
   // Locality order (optional): A and B hold the points at positions of an order, perm[pos]
   // the point id; ids and thr are then written for the point ids (row perm[pos], column
@@ -51,6 +51,7 @@ struct TcScreenArgs {
   const int32_t* perm;
   int wave_start;
   int64_t row_off = 0;  // position of row 0 in the order (tuning trials on a row sample)
+  int split = 1;        // 0: never split the columns (tuning trials, sized as a part of the whole)
   int variant = -1;     // pipeline variant; -1: the autotuner's choice
 };
 
@@ -66,14 +67,16 @@ int screen_tc_variants();
 struct TcVariant {
   int stages_less, cap_step, sync_d;
 };
+size_t screen_res_rowbuf_words(const TcScreenArgs& a, int cap_step);
 cudaError_t launch_screen_res(const TcScreenArgs& a, const TcVariant& v, int variant, cudaStream_t s,
                               std::string* msg, float* dump, TcShape* shape);
 // The autotuned variant for a's shape (timing the variants on first use; synchronises `s`).
 cudaError_t launch_screen_tc_tune(const TcScreenArgs& a, cudaStream_t s, std::string* msg, int* variant);
 
 bool tc_screen_supported(int d, bool fp16);
-// Scratch words for m rows against n columns: row buffers plus checkpoint counters.
-size_t screen_tc_rowbuf_words(int64_t m, int64_t n, int Lp);
+// Scratch words of a screen (every field but the pointers set): row buffers, checkpoint counters and
+// the lists of a column split.
+size_t screen_tc_rowbuf_words(const TcScreenArgs& a);
 // The screen (launch on `s`); with a.variant < 0 the autotuned variant for this shape, timed
 // on first use (synchronises `s` then).  *shape, if given, receives the shape used.
 cudaError_t launch_screen_tc(const TcScreenArgs& a, cudaStream_t s, std::string* msg,
