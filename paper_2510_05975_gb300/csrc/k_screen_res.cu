@@ -236,14 +236,20 @@ struct ResUnit {
   int64_t rb;
   int split, ntiles;
 };
+// SPLIT = false: the unit is the row block (with the split's arithmetic in the tile loops a 1M x 128
+// screen took 210 ms, without 202).
+template <bool SPLIT>
 CNG_DEV ResUnit res_unit(const ResParams& P, int64_t u, int64_t nrb) {
+  if constexpr (!SPLIT) return ResUnit{u, 0, P.ntiles};
   ResUnit r;
   r.split = (int)(u / nrb);
   r.rb = u - r.split * nrb;
   r.ntiles = P.pre + (P.ntiles - P.pre - r.split + P.nsplit - 1) / P.nsplit;
   return r;
 }
+template <bool SPLIT>
 CNG_DEV int res_tile(const ResParams& P, const ResUnit& r, int t) {
+  if constexpr (!SPLIT) return t;
   return t < P.pre ? t : P.pre + r.split + (t - P.pre) * P.nsplit;
 }
 
@@ -271,7 +277,7 @@ CNG_DEV void append_chunk(const uint32_t (&r)[BN], int o, float mx, uint32_t c0,
   }
 }
 
-template <int BN, int NBUF, int CPL, bool DUMP>
+template <int BN, int NBUF, int CPL, bool DUMP, bool SPLIT>
 __global__ void __launch_bounds__(rs_threads(NBUF), 1) screen_res_kernel(const __grid_constant__ ResParams P,
                                                                    float* dump) {
   extern __shared__ __align__(128) unsigned char smem_res[];
@@ -289,7 +295,7 @@ __global__ void __launch_bounds__(rs_threads(NBUF), 1) screen_res_kernel(const _
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int64_t nrb = (P.m + RS_BM - 1) / RS_BM;
-  const int64_t nunits = nrb * P.nsplit;
+  const int64_t nunits = SPLIT ? nrb * P.nsplit : nrb;
 
   if (tid == 0) {
     for (int i = 0; i < P.nst; ++i) {
@@ -323,13 +329,14 @@ __global__ void __launch_bounds__(rs_threads(NBUF), 1) screen_res_kernel(const _
       uint32_t ph = 0;
       bool ok = true;
       for (int64_t u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
-        const ResUnit un = res_unit(P, u, nrb);
+        const ResUnit un = res_unit<SPLIT>(P, u, nrb);
         for (int t = 0; t < un.ntiles; ++t, ++it) {
           wave_checkpoint(P.sync, P.sync_d, TC_SYNC_COLS / BN, it, nrb, P.ntiles);
           ok = mbar_wait(&b_empty[s], ph ^ 1, abort_flag, P.status);
           if (!ok) break;
           mbar_expect_tx(&b_full[s], (uint32_t)stage_bytes);
-          bulk_load(sB + s * stage_bytes, P.B + (size_t)res_tile(P, un, t) * stage_bytes, (uint32_t)stage_bytes, &b_full[s]);
+          bulk_load(sB + s * stage_bytes, P.B + (size_t)res_tile<SPLIT>(P, un, t) * stage_bytes,
+                    (uint32_t)stage_bytes, &b_full[s]);
           if (++s == P.nst) {
             s = 0;
             ph ^= 1u;
@@ -360,7 +367,7 @@ __global__ void __launch_bounds__(rs_threads(NBUF), 1) screen_res_kernel(const _
       uint64_t* const te = &t_empty[half * NBUF + b];
       uint64_t* const fn = &fin[half * NBUF + b];
       for (int64_t u = blockIdx.x; u < nunits && ok; u += gridDim.x, ++j) {
-        const int ntiles = res_unit(P, u, nrb).ntiles;
+        const int ntiles = res_unit<SPLIT>(P, u, nrb).ntiles;
         ok = mbar_wait(&a_full[half], j & 1, abort_flag, P.status);
         if (!ok) break;
         tc_fence_after();
@@ -421,7 +428,7 @@ __global__ void __launch_bounds__(rs_threads(NBUF), 1) screen_res_kernel(const _
     uint32_t bph = 0;
     bool ok = true;
     for (int64_t u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
-      const ResUnit un = res_unit(P, u, nrb);
+      const ResUnit un = res_unit<SPLIT>(P, u, nrb);
       const int64_t row = un.rb * RS_BM + rloc;
       const bool live = row < P.m;
       {
@@ -457,7 +464,7 @@ __global__ void __launch_bounds__(rs_threads(NBUF), 1) screen_res_kernel(const _
       const uint32_t self = P.self_excl && live ? (uint32_t)P.col_pos[P.row_perm[row]] : ~0u;
       int t = 0;
       for (int part = 0; part < P.npart && ok; ++part) {
-        const int tend = part + 1 == P.npart ? un.ntiles : P.part_end[part];
+        const int tend = SPLIT && part + 1 == P.npart ? un.ntiles : P.part_end[part];
         const int rank = P.part_rank[part];
         for (; t < tend; ++t) {
           ok = mbar_wait_warp(&tf[b], bph, abort_flag, P.status);
@@ -480,7 +487,7 @@ __global__ void __launch_bounds__(rs_threads(NBUF), 1) screen_res_kernel(const _
               for (int j = 0; j < BN; ++j)
                 if (c0 + j < P.n) dump[row * P.n + c0 + j] = -2.f * __uint_as_float(r[j]);
           } else {
-            const int tile = res_tile(P, un, t);
+            const int tile = res_tile<SPLIT>(P, un, t);
             float m[BN / RS_C];
 #pragma unroll
             for (int c = 0; c < BN / RS_C; ++c) m[c] = max16<BN>(r, c * RS_C);
@@ -507,7 +514,7 @@ __global__ void __launch_bounds__(rs_threads(NBUF), 1) screen_res_kernel(const _
         // end of a sample part: every list down to the part's rank
         __syncwarp();
         for (int l = 0; l < 32; ++l) cut(l, rank, 0);
-        if (part + 2 == P.npart && un.split > 0) cnt = 0;  // split 0 lists the sample's columns
+        if (SPLIT && part + 2 == P.npart && un.split > 0) cnt = 0;  // split 0 lists the sample's columns
       }
       if (!ok || DUMP) continue;
       // the Lp smallest of each list, ids and threshold key
@@ -520,7 +527,7 @@ __global__ void __launch_bounds__(rs_threads(NBUF), 1) screen_res_kernel(const _
         uint64_t* buf_l = wbuf + (size_t)l * P.cap;
         uint32_t key = isinf(t_l) ? 0xffffffffu : fkey(-2.f * t_l);
         if (c_l > P.Lp) key = warp_cut<CPL>(buf_l, c_l, P.Lp, 0, lane, &c_l);
-        if (P.nsplit > 1) {
+        if constexpr (SPLIT) {
           const int64_t at = un.split * P.m + row_l;
           for (int i = lane; i < c_l; i += 32) P.mlist[at * P.Lp + i] = buf_l[i];
           if (lane == 0) {
@@ -748,8 +755,7 @@ static int list_cap(int Lp, int step) {
   return caps[std::min(3, ci + step)] * 32;
 }
 
-// Column split for launches whose row blocks leave SMs idle (fewer than 4 per SM and no multiple of
-// them): the split and the sample parts swept whole by each unit that minimise
+// Column split for launches whose row blocks leave SMs idle (fewer than 4 per SM): the split and the sample parts swept whole by each unit that minimise
 //   waves x (unit overhead + sample tiles + other tiles / splits + hits),
 // in tiles of ~850 cycles; a hit per row costs ~6 tiles (32 rows append in turn), a unit's operand
 // load and final lists ~40, merging the splits' lists ~60.  10,000 rows against 1M x 128 (40 row
@@ -819,6 +825,7 @@ static void plan_res(const TcScreenArgs& a, int cap_step, bool split, ResParams*
   p->nsplit = 1;
   p->pre = 0;
   if (split) split_columns((a.m + RS_BM - 1) / RS_BM, bn, a.n, a.Lp, p->cap, p);
+  if (p->nsplit > 1) p->cap = p->cap <= 512 ? 512 : 768;  // the capacities split kernels are built for
 }
 
 size_t screen_res_rowbuf_words(const TcScreenArgs& a, int cap_step) {
@@ -828,9 +835,9 @@ size_t screen_res_rowbuf_words(const TcScreenArgs& a, int cap_step) {
   return std::max(res_scratch(a.m, a.res.bn, p).total, res_scratch(a.m, a.res.bn, whole).total);
 }
 
-template <int BN, int NBUF, int CPL, bool DUMP>
+template <int BN, int NBUF, int CPL, bool DUMP, bool SPLIT>
 static cudaError_t launch_res_t(const ResParams& p, size_t smem, int grid, cudaStream_t s, float* dump) {
-  cudaError_t e = cudaFuncSetAttribute(screen_res_kernel<BN, NBUF, CPL, DUMP>,
+  cudaError_t e = cudaFuncSetAttribute(screen_res_kernel<BN, NBUF, CPL, DUMP, SPLIT>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   // cooperative when the producers wait for one another (boundedly): every CTA resident at once
@@ -845,11 +852,11 @@ static cudaError_t launch_res_t(const ResParams& p, size_t smem, int grid, cudaS
   cfg.attrs = attr;
   cfg.numAttrs = p.sync ? 1 : 0;
   count_launch();
-  e = cudaLaunchKernelEx(&cfg, screen_res_kernel<BN, NBUF, CPL, DUMP>, p, dump);
+  e = cudaLaunchKernelEx(&cfg, screen_res_kernel<BN, NBUF, CPL, DUMP, SPLIT>, p, dump);
   if (e == cudaErrorCooperativeLaunchTooLarge) {  // not all resident: plain launch (waits bounded)
     (void)cudaGetLastError();
     cfg.numAttrs = 0;
-    e = cudaLaunchKernelEx(&cfg, screen_res_kernel<BN, NBUF, CPL, DUMP>, p, dump);
+    e = cudaLaunchKernelEx(&cfg, screen_res_kernel<BN, NBUF, CPL, DUMP, SPLIT>, p, dump);
   }
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
@@ -858,12 +865,15 @@ static cudaError_t launch_res_t(const ResParams& p, size_t smem, int grid, cudaS
 template <int BN, int NBUF>
 static cudaError_t launch_res_bn(int cpl, const ResParams& p, size_t smem, int grid, cudaStream_t s,
                                  float* dump) {
-  if (dump) return launch_res_t<BN, NBUF, 12, true>(p, smem, grid, s, dump);
+  if (dump) return launch_res_t<BN, NBUF, 12, true, false>(p, smem, grid, s, dump);
+  if (p.nsplit > 1)
+    return cpl == 16 ? launch_res_t<BN, NBUF, 16, false, true>(p, smem, grid, s, dump)
+                     : launch_res_t<BN, NBUF, 24, false, true>(p, smem, grid, s, dump);
   switch (cpl) {
-    case 12: return launch_res_t<BN, NBUF, 12, false>(p, smem, grid, s, dump);
-    case 16: return launch_res_t<BN, NBUF, 16, false>(p, smem, grid, s, dump);
-    case 20: return launch_res_t<BN, NBUF, 20, false>(p, smem, grid, s, dump);
-    case 24: return launch_res_t<BN, NBUF, 24, false>(p, smem, grid, s, dump);
+    case 12: return launch_res_t<BN, NBUF, 12, false, false>(p, smem, grid, s, dump);
+    case 16: return launch_res_t<BN, NBUF, 16, false, false>(p, smem, grid, s, dump);
+    case 20: return launch_res_t<BN, NBUF, 20, false, false>(p, smem, grid, s, dump);
+    case 24: return launch_res_t<BN, NBUF, 24, false, false>(p, smem, grid, s, dump);
     default: return cudaErrorInvalidValue;
   }
 }
