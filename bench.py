@@ -327,7 +327,7 @@ SCREEN_DRAM_BYTES = {("sift1m", "2fde0dbd24a93892"): 18.55e9 + 20.29e9}
 def screen_digest() -> str:
     import hashlib
 
-    path = os.path.join(ROOT, "paper_2510_05975_gb300", "csrc", "k_screen_tc.cu")
+    path = os.path.join(ROOT, "paper_2510_05975_gb300", "csrc", "k_screen_res.cu")
     with open(path, "rb") as f:
         return hashlib.sha256(f.read()).hexdigest()[:16]
 

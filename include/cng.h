@@ -129,7 +129,7 @@ typedef struct {
   double ms_total, ms_prep, ms_entry, ms_screen, ms_rerank, ms_prune, ms_merge, ms_connect;
   int64_t n_edges;            /* edges of the final graph */
   int64_t cert_fail_rows;     /* rows whose screened list could not be certified, rescanned */
-  int64_t order_ties;         /* candidate-order near-ties re-decided in FP64 */
+  int64_t order_ties;         /* candidate-order near-ties re-decided beyond FP32 */
   int64_t rule_ties;          /* pruning comparisons re-decided in FP64 */
   int64_t merge_repruned;     /* nodes whose merged list exceeded R and was pruned again */
   int64_t merge_max_list;     /* largest merged candidate set */
@@ -145,7 +145,7 @@ typedef struct {
                                  ms_rerank then time G0's exact K-NN, when the library builds it) */
   int32_t screen_variant;     /* tensor-core screen: the pipeline variant used, its operand */
   int32_t screen_stages;      /* stages, row-buffer capacity (entries per row) and checkpoint */
-  int32_t screen_cap;         /* lag (windows of 256 column tiles); -1 for the FP32 screen */
+  int32_t screen_cap;         /* lag (windows of 32,768 columns); -1 for the FP32 screen */
   int32_t screen_sync;
   int32_t prune_path;         /* phase-2b sweep: 0 float rows (SIMT), 1 8-bit rows (dp4a SIMT),
                                  2 8-bit rows, candidate-pair Gram tile on the tensor cores,

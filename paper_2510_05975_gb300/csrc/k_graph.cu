@@ -1058,7 +1058,8 @@ merge_kernel(const T* __restrict__ Xs, int64_t n, int d, int dpad, const int32_t
 // instruction, 16 in flight) and orders it by (D(p,.), id); sets of at most R entries become rows at
 // once, the others are listed.  Nodes with more entries go to mid_list for merge_kernel.  Bound by the
 // rows' gathers; a CTA per node with its barriers and 100 KB of shared memory (merge_kernel) kept 16
-// warps on an SM, this 32 or more.  1M x 96 (R = 48): 45 -> 16 ms; 1M x 128 FP16: 31 -> 11 ms.
+// warps on an SM, this 32 or more.  The whole merge (these lists and the re-prune): 1M x 96, R = 48,
+// 101 -> 60 ms; 1M x 128 FP16, re-pruned on the Gram tile, 94 -> 12.4 ms.
 constexpr int ML_CAP = 256;
 constexpr int ML_WARPS = 4;
 constexpr size_t ml_warp_bytes(int dpad) {

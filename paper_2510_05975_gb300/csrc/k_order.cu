@@ -1,14 +1,13 @@
 // k_order.cu -- locality order of the point set for the tensor-core screen (an engineering
 // addition; the paper has no counterpart).
 //
-// The screen keeps, for every row, the L' smallest screened scores seen so far; a 32-column
-// chunk in which some row of a warp scores below its current threshold takes the slow append
-// path.  With the columns swept in input order (random with respect to each row) the
-// thresholds fall slowly and a large share of the chunks take that path.  Sorting the points
-// into a k-d order, and starting each wave of row blocks at its own position in that order,
-// brings most of a row's nearest columns first, so its threshold is tight early and most later
-// chunks take the fast path.  The order changes nothing but speed: the screen only proposes
-// candidates, and the rerank certifies them exactly (rows it cannot certify are rescanned).
+// Rows of a warp of the screen's epilogue whose near columns agree append in the same column tiles,
+// so most tiles have no append for the warp; sorting the points into a k-d order brings such rows
+// together.  The resident kernel (k_screen_res.cu) sweeps the columns in a sampled order (below, its
+// parts each in k-d order), the streamed one in k-d order with each wave of row blocks starting at its
+// own position, which brings most of a row's nearest columns first.  The order changes nothing but
+// speed: the screen only proposes candidates, and the rerank certifies them exactly (rows it cannot
+// certify are rescanned).
 //
 // The order: 16 random +-1 projections of every point; then, level by level, every segment of
 // the current order is sorted (stably) by the projection with the largest variance over a
