@@ -338,6 +338,7 @@ static cng_status run_knn(const KnnInputs& in, int32_t* out_ids, float* out_dist
     sm.normmax = in.normmax;
     // K terms, 2^-23 per add (the norm pieces among them when they are part of the operands)
     sm.acc_err = (float)(in.res.kt > 0 ? in.res.kt + 16 : in.kpad + 8) * 1.1920929e-7f;
+    sm.abs_err = in.res.kt > 0 && in.tc_fp16 ? RES_PIECE_ERR : 0.f;
     sm.scale2 = in.scale2;
   } else {
     int cpl = 0;
@@ -393,13 +394,13 @@ struct Prepared {
   PrepStats st{};
 };
 
-// Tensor-core operand scale: 1 for integer data with |x| <= 2048 (exact in FP16) and for FP16
-// input; otherwise the power of two that puts max |s x| in (4096, 8192], which keeps the FP16
-// operands clear of overflow and of the subnormal range (relative rounding 2^-11).
+// Tensor-core operand scale: 1 for integer data with |x| <= 2048 (exact in FP16); otherwise the
+// power of two that puts max |s x| in (4096, 8192], which keeps the FP16 operands clear of overflow
+// and of the subnormal range (relative rounding 2^-11) and their norms far above the resolution of
+// the resident kernel's norm pieces.  FP16 input is only scaled up, which is exact.
 static cng_status operand_scale(const void* const* pts, const int64_t* ns, int count, int dtype,
                                 int d, float* scale, cudaStream_t s) {
   *scale = 1.f;
-  if (dtype != CNG_F32) return CNG_OK;
   DevPool pool;
   uint32_t* dev;
   CK(pool.alloc(&dev, 2));
@@ -414,7 +415,7 @@ static cng_status operand_scale(const void* const* pts, const int64_t* ns, int c
   if (!host[1] && amax <= 2048.f) return CNG_OK;
   if (!(amax > 0.f) || !std::isfinite(amax)) return CNG_OK;
   const int e = (int)std::ceil(std::log2((double)amax));
-  *scale = (float)std::ldexp(1.0, 13 - e);
+  *scale = (float)std::ldexp(1.0, dtype == CNG_F32 ? 13 - e : std::max(13 - e, 0));
   return CNG_OK;
 }
 
@@ -443,8 +444,8 @@ static cng_status prepare(DevPool& pool, const void* pts_dev, int dtype, int64_t
   PrepStats init{};
   init.vmin_key = 0xffffffffu;
   CK(cudaMemcpyAsync(dst, &init, sizeof(init), cudaMemcpyHostToDevice, s));
-  CK(launch_prep(pts_dev, dtype, n, d, dpad, out->xs, xb_bf, xb_h, kpad, out->nb, out->rb,
-                 dtype == CNG_F32 ? scale : 1.f, dst, s));
+  CK(launch_prep(pts_dev, dtype, n, d, dpad, out->xs, xb_bf, xb_h, kpad, out->nb, out->rb, scale,
+                 dst, s));
   CK(cudaMemcpyAsync(&out->st, dst, sizeof(PrepStats), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   return CNG_OK;

@@ -76,6 +76,7 @@ struct ScreenModel {
   const float* rb;   // kind 1: ||x_b - x|| per point
   float rbmax;       // kind 1: max rb
   float acc_err;     // kind 1: absolute accumulation error bound per unit of (||x||+||y||)^2
+  float abs_err;     // kind 1: further error of a score, whatever the norms
   float normmax;     // kind 1: max ||x_b||
   float scale2;      // kind 1: the operands are x_b ~ s x; scores are in units of s^2 (a power of 4)
 };

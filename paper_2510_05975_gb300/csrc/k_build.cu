@@ -493,7 +493,7 @@ CNG_DEV bool rerank_sort_certify(uint64_t* keys, int P2, int cnt, int64_t row, i
         ok = (sc + nx) > dLs;
       } else {
         float nrm = sqrtf(fmaxf(nx, 0.f));
-        float eacc = sm.acc_err * (nrm + sm.normmax) * (nrm + sm.normmax);
+        float eacc = sm.acc_err * (nrm + sm.normmax) * (nrm + sm.normmax) + sm.abs_err;
         float db = sqrtf(fmaxf(sc + nx - eacc, 0.f)) - (sm.rb[row] + sm.rbmax);
         ok = db > 0.f && db * db > dLs * (1.f + 2.f * band);
       }

@@ -6,8 +6,9 @@
 // and certifies the list.
 //
 // Operands.  Each operand row has kt = d + 6 elements rounded up to 16: the d coordinates, then
-// six norm pieces.  A column holds p_0..p_5 with sum c_i p_i = ||y_b||^2 / 2 to about 32 bits, a
-// row holds the constants -c_i, so the accumulator is a = <x_b, y_b> - ||y_b||^2 / 2 = -s / 2 and
+// six norm pieces.  A column holds p_0..p_5 with sum c_i p_i = ||y_b||^2 / 2 to max(2^-35 of it,
+// 2^-25) in FP16 (operands are scaled so that the largest coordinate exceeds 4096 unless they are
+// integers, and the certification counts the absolute part) and to 2^-48 of it in BF16, a row holds the constants -c_i, so the accumulator is a = <x_b, y_b> - ||y_b||^2 / 2 = -s / 2 and
 // the epilogue only compares it with the row's threshold (an FMA and a shared-memory norm load per
 // score in the epilogue's fast path cost more than the extra 16 K elements of the MMA).  Integer
 // operands with ||x||^2 < 2^23 stay exact: pieces, products and sums are multiples of 1/2 below
@@ -671,7 +672,8 @@ __global__ void __launch_bounds__(256) tile_image_kernel(const uint32_t* __restr
 }
 
 // Piece scales: FP16 pieces reach 65504 and resolve 2^-24 of their scale, so 2^15 four times
-// covers ||y_b||^2 / 2 up to RES_NORM_MAX and 2^9, 1 take the remainder; BF16 pieces have FP32's
+// covers ||y_b||^2 / 2 up to RES_NORM_MAX and 2^9, 1 take the remainder, down to 2^-25
+// (RES_PIECE_ERR); BF16 pieces have FP32's
 // range, so each takes 8 bits of the remainder at scale 1.
 static AuxScale aux_scales(bool fp16) {
   AuxScale a;

@@ -14,6 +14,10 @@ namespace cng {
 constexpr int RES_AUX = 6;
 constexpr int RES_PARTS = 4;                                // parts of the sampled column order
 constexpr float RES_NORM_MAX = 4.f * 65504.f * 32768.f;     // largest ||y_b||^2 / 2 the pieces hold
+// FP16 pieces hold ||y_b||^2 / 2 to max(2^-25, 2^-35 of it): the relative part is far below the
+// accumulation error, the absolute one (twice that in a score; a factor 2 more is left) is not for
+// operands with norms below about 0.03, which the operand scale avoids.
+constexpr float RES_PIECE_ERR = 1.1920929e-7f;              // 2^-23
 struct ResShape {
   int d = 0, kt = 0, bn = 0;
 };
