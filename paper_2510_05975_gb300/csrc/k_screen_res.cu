@@ -170,11 +170,13 @@ CNG_DEV float max16(const uint32_t (&r)[BN], int o) {
 // is found first: moves them to the front of buf and returns the largest kept score key; *kept =
 // their number.  Every dropped key lies at or above every kept one.  Bisection on the 32-bit score
 // keys with one warp reduction per step; with the cut inside a run of equal keys the first of
-// them in buffer order are kept.  cnt <= 32 CPL, cnt > need.
+// them in buffer order are kept.  cnt <= 32 CPL, cnt > need.  The other lanes' appends to buf are
+// ordered before its loads here (votes and shuffles order no memory).
 template <int CPL>
 CNG_DEV uint32_t warp_cut(uint64_t* buf, int cnt, int need, int slack, int lane, int* kept) {
   uint64_t e[CPL];
   uint32_t k[CPL];
+  __syncwarp();
   uint32_t lo = 0xffffffffu, hi = 0u;
 #pragma unroll
   for (int i = 0; i < CPL; ++i) {
