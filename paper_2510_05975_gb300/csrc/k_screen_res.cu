@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(rs_threads(NBUF), 1) screen_res_kernel(const _
       mbar_init(&t_full[i], 1);
       mbar_init(&t_empty[i], 4);
     }
-    for (int i = 0; i < 2; ++i) mbar_init(&a_full[i], 4);
+    for (int i = 0; i < 2; ++i) mbar_init(&a_full[i], 4 + NBUF);  // the half's warps and issuers
     for (int i = 0; i < 2 * NBUF; ++i) mbar_init(&fin[i], 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -371,6 +371,10 @@ __global__ void __launch_bounds__(rs_threads(NBUF), 1) screen_res_kernel(const _
       uint64_t* const fn = &fin[half * NBUF + b];
       for (int64_t u = blockIdx.x; u < nunits && ok; u += gridDim.x, ++j) {
         const int ntiles = res_unit<SPLIT>(P, u, nrb).ntiles;
+        // An issuer takes part in the phase it waits for: with a single column tile a unit leaves one
+        // buffer's issuer without work, and the next unit's phase could otherwise complete before
+        // that issuer has seen this one (a parity wait cannot tell the two apart).
+        mbar_arrive(&a_full[half]);
         ok = mbar_wait(&a_full[half], j & 1, abort_flag, P.status);
         if (!ok) break;
         tc_fence_after();
@@ -893,7 +897,13 @@ cudaError_t launch_screen_res(const TcScreenArgs& a, const TcVariant& v, int var
   plan_res(a, v.cap_step, a.split && !dump, &p);
   const int stage_bytes = bn * kt * 2;
   const int fixed = (2 * RS_MAXST + 14) * 8 + 16;
+  // at least 4: an issuer sees every phase of its stages (an even number of them), or (5) reaches a
+  // stage's next phase only after the epilogue has read the tile of the one it skipped
   p.nst = std::min(RS_MAXST, (226 * 1024 - fixed) / stage_bytes) - v.stages_less;
+  if (p.nst < 4) {
+    if (msg) *msg = "shared memory too small for four column tiles; ";
+    return cudaErrorInvalidValue;
+  }
   if (p.cap < a.Lp + 128) {
     if (msg) *msg = "screened list too long; ";
     return cudaErrorInvalidValue;
