@@ -7,7 +7,7 @@
 // whose unsigned order is the (FP32 D^2, id) order.  FP32 decides every comparison that lies
 // outside the relative band; the rest is Alg. 1's order by the canonical FP64 distance:
 //   after the new points of a hop are merged, every two neighbours of the queue (and the last kept
-//   against the first dropped) that lie within the band and are not both `decided` get their
+//   against each dropped one) that lie within the band and are not both `decided` get their
 //   squared distance to within DD_EPS (warp_sqdist_dd, ~120 FP32 instructions of the warp; one
 //   lane's FP64 sum holds the SM's FP64 pipe for ~80 d cycles, which bounded the searches of
 //   unit-norm data), and its FP32 rounding replaces the key's D^2.  So two decided entries more
@@ -185,7 +185,7 @@ __device__ __noinline__ bool canon_before(uint64_t a, uint64_t b, const float* q
   return da < db || (da == db && fk_id(a) < fk_id(b));
 }
 
-// Settles the near-ties of the queue qm and of its end against the dropped keys (one per lane); dec
+// Settles the near-ties of the queue qm and of its end against all dropped keys (one per lane); dec
 // counts the entries decided, moves the key moves of the query.  Returns false if the query has to
 // be left to the general kernel.  A call of its own, with the queue through (local) memory: it is
 // rare, and inlined it left the warp in pieces for the rest of the query (20 of 32 lanes to an
@@ -210,16 +210,11 @@ __device__ __noinline__ bool fq_fix(uint64_t* qm, uint64_t drop, const float* qv
       mark[s] = q[s] != KINF && (fk_near(q[s], nx, band) || (!first && fk_near(pv, q[s], band)));
       any |= mark[s];
     }
-    // the last kept key against the smallest dropped one
+    // the last kept key against every dropped one: while undecided, any of those within the band may
+    // come before it
     const uint64_t last = __shfl_sync(FULL, q[QS - 1], 31);
-    uint64_t dmin = drop;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const uint64_t y = __shfl_xor_sync(FULL, dmin, o);
-      dmin = y < dmin ? y : dmin;
-    }
-    const int dsrc = __ffs(__ballot_sync(FULL, drop == dmin)) - 1;
-    const bool edge = last != KINF && dmin != KINF && (dmin < last || fk_near(last, dmin, band));
+    const bool dnear = last != KINF && drop != KINF && (drop < last || fk_near(last, drop, band));
+    const bool edge = __any_sync(FULL, dnear);
     if (edge && lane == 31) mark[QS - 1] = true;
     if (__any_sync(FULL, any || edge)) {
 #pragma unroll
@@ -233,12 +228,29 @@ __device__ __noinline__ bool fq_fix(uint64_t* qm, uint64_t drop, const float* qv
           if (lane == l) q[s] = k;
         }
       }
-      if (edge) {  // the dropped key too; the smaller of the two stays
-        const uint64_t d1 = fk_decide(dmin, qv, X, dpad, d, lane), l1 = __shfl_sync(FULL, q[QS - 1], 31);
-        if (lane == dsrc) drop = d1 < l1 ? l1 : d1;
-        if (lane == 31 && d1 < l1) q[QS - 1] = d1;
+      unsigned db = __ballot_sync(FULL, dnear && !(drop & 2));
+      while (db) {
+        const int l = __ffs(db) - 1;
+        db &= db - 1;
+        const uint64_t k = fk_decide(__shfl_sync(FULL, drop, l), qv, X, dpad, d, lane);
+        if (lane == l) drop = k;
       }
       fq_settle<QS>(q, lane);
+      // dropped keys that came out below the last kept one change places with it: each enters at most
+      // once, as the last key only falls
+      for (;;) {
+        const uint64_t lk = __shfl_sync(FULL, q[QS - 1], 31);
+        uint64_t dmin = drop;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          const uint64_t y = __shfl_xor_sync(FULL, dmin, o);
+          dmin = y < dmin ? y : dmin;
+        }
+        if (lk == KINF || dmin >= lk) break;
+        if (lane == __ffs(__ballot_sync(FULL, drop == dmin)) - 1) drop = lk;
+        if (lane == 31) q[QS - 1] = dmin;
+        fq_settle<QS>(q, lane);
+      }
       continue;
     }
     // decided neighbours within CLOSE_STEPS: their keys have to be in the FP64 order
@@ -259,13 +271,19 @@ __device__ __noinline__ bool fq_fix(uint64_t* qm, uint64_t drop, const float* qv
       }
     }
     wrong = moved != 0;
-    if (!wrong && fk_close(last, dmin) && !canon_before(last, dmin, qv, X, dpad, d, lane)) {
-      // the smallest dropped point belongs in the queue, the last one out of it
-      wrong = true;
-      lost |= (last >> 33) != (dmin >> 33);
-      ++moved;
-      if (lane == 31) q[QS - 1] = dmin;
-      if (lane == dsrc) drop = last + STEP;
+    if (!wrong) {
+      unsigned cb = __ballot_sync(FULL, fk_close(last, drop));
+      while (cb) {
+        const int l = __ffs(cb) - 1;
+        cb &= cb - 1;
+        const uint64_t kd = __shfl_sync(FULL, drop, l);
+        if (canon_before(last, kd, qv, X, dpad, d, lane)) continue;
+        // the dropped point belongs in the queue, the last one out of it for good
+        wrong = true;
+        if (lane == 31) q[QS - 1] = kd;
+        if (lane == l) drop = KINF;
+        break;
+      }
     }
     moves += moved;
     if (lost || moves > CLOSE_STEPS) break;
