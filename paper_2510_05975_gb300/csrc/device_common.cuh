@@ -112,6 +112,14 @@ CNG_DEV double warp_sqdist_dd(const TA* x, const TB* y, int d, int lane) {
   return v >= 1e-25 && v <= 1e30 ? v : __longlong_as_double(0x7ff8000000000000ll);
 }
 
+// Whether two rows are equal in all coordinates; all lanes take part.
+template <typename TA, typename TB>
+CNG_DEV bool warp_rows_equal(const TA* x, const TB* y, int d, int lane) {
+  bool ne = false;
+  for (int i = lane; i < d; i += 32) ne |= to_f(x[i]) != to_f(y[i]);
+  return !__any_sync(FULL, ne);
+}
+
 // Whether two values of warp_sqdist_dd leave the canonical order open.
 CNG_DEV bool dd_open(double a, double b) { return !(fabs(a - b) > DD_EPS * fmax(fabs(a), fabs(b))); }
 

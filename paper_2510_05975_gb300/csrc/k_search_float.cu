@@ -10,13 +10,14 @@
 //   against each dropped one) that lie within the band and are not both `decided` get their
 //   squared distance to within DD_EPS (warp_sqdist_dd, ~120 FP32 instructions of the warp; one
 //   lane's FP64 sum holds the SM's FP64 pipe for ~80 d cycles, which bounded the searches of
-//   unit-norm data), and its FP32 rounding replaces the key's D^2.  So two decided entries more
-//   than one FP32 step apart are in the FP64 order, and an entry's key stays within the band's
-//   error model (2^-24 instead of 2.6e-6).  Two decided neighbours closer than that are compared by
-//   those distances (in FP64 within DD_EPS); where two equal roundings are not in that order, the
-//   later one's key moves up by one FP32 step.  A query that needs more than CLOSE_STEPS such moves, or whose near-ties do
-//   not settle in a few rounds, is left to the general kernel (k_search.cu): one such query takes
-//   longer there than the whole batch here, so these have to be (and are) rare.
+//   unit-norm data), and its FP32 rounding replaces the key's D^2.  Two decided neighbours within
+//   CLOSE_STEPS FP32 steps, one of them new to its place, are compared by those values -- by id where
+//   their rows are the same, in FP64 (one entry per lane) where the values lie within DD_EPS -- and
+//   while they are not in that order the later one's key moves up by one FP32 step.  No key moves
+//   further than CLOSE_STEPS from its rounding, so decided entries further apart than that are in the
+//   FP64 order, and an entry's key stays within the band's error model (2^-20.3; an FP32 sum
+//   2^-18.6).  A query that needs more, whose near-ties do not settle in FIX_ROUNDS rounds or take
+//   FP64 sums in many hops, is left to the general kernel (k_search.cu).
 // So the queue, and with it every hop, id and hop count, equals the FP64 definition of Alg. 1.
 //
 // What bounds it: the latency of a hop's dependent steps -- row loads, filter, sort, merge -- over
@@ -26,9 +27,9 @@
 // each), a register sort, a register merge and one neighbour comparison per slot.
 // The FP32 distances are those of the general kernel bit for bit (same sums in the same order).
 //
-// Measured (start: the general kernel alone): 10,000 queries on 1M x 96 FP32 rows, L = 24: 2.36 -> 0.81
-// ms (4.8 TB/s of rows); 100,000 on 1M x 128 FP16 rows, L = 64: 31.4 -> 13.0 ms; learned stop, 500k x
-// 128 FP16, L = 192: 12.3 -> 8.4 ms; the phase-4 searches of 50k x 960 rows, L = 128: 180 -> 28 ms.
+// Measured (start: the general kernel alone): 10,000 queries on 1M x 96 FP32 rows, L = 24: 2.36 -> 0.82
+// ms (4.8 TB/s of rows); 100,000 on 1M x 128 FP16 rows, L = 64: 31.4 -> 13.2 ms; learned stop, 500k x
+// 128 FP16, L = 192: 12.3 -> 7.6 ms; the phase-4 searches of 50k x 960 rows, L = 128: 180 -> 28 ms.
 #include "launch_count.h"
 #include "cng_internal.h"
 #include "device_common.cuh"
@@ -40,11 +41,17 @@ namespace cng {
 namespace {
 
 constexpr uint64_t KINF = ~0ull;
-constexpr int FIX_ROUNDS = 48;  // near-tie rounds of a hop before a query is left to the general kernel
-// Key moves of a query at most, and the FP32 steps within which decided neighbours are compared
-// again: a key is at most CLOSE_STEPS steps above its rounding, so neighbours further apart than that
-// are in order.
-constexpr int CLOSE_STEPS = 3;
+constexpr int FIX_ROUNDS = 64;   // near-tie rounds of a hop before a query is left to the general kernel
+constexpr int CLOSE_STEPS = 6;   // FP32 steps a key may lie above its rounding
+// FP64 sums (plus three in two hops for queues of up to 64 entries, one in two for longer ones, whose
+// hops take more of them) after which a query is left to the general kernel, which keeps an entry's
+// FP64 distance for the query's later hops.  Only data whose distances tie to the last FP64 bits comes
+// near it.  A round of moves that follows such a sum counts as MOVE_SUMS more.  2,000 queries on 20,000
+// rows of two levels, d = 64, the general kernel alone / this file without the limit / with it: L = 32
+// 3.6 / 2.8 / 2.8 ms, L = 64 6.1 / 5.6 / 5.7, L = 256 24.9 / 55 / 27; three levels, d = 96, L = 64 8.5 /
+// 17 / 9.3, L = 128 15.3 / 44 / 16.
+constexpr int FP64_SUMS = 8;
+constexpr int MOVE_SUMS = 2;
 
 CNG_DEV uint64_t fk_make(float d2, int32_t id) {
   return ((uint64_t)__float_as_uint(d2) << 33) | ((uint64_t)(uint32_t)id << 2);
@@ -117,39 +124,112 @@ CNG_DEV uint64_t fq_merge(uint64_t (&q)[QS], uint64_t kdesc, int lane) {
   return drop;
 }
 
-// Sorts a nearly sorted queue (odd-even transposition until nothing is out of order).
+// Per-lane flags (bit s: the entry q[s]) of the entries after / before this lane's (0 past the ends).
 template <int QS>
-CNG_DEV void fq_settle(uint64_t (&q)[QS], int lane) {
+CNG_DEV unsigned fq_next_bits(unsigned f, int lane) {
+  const unsigned nx = __shfl_down_sync(FULL, f, 1), first = __shfl_sync(FULL, f, 0) >> 1;
+  return lane == 31 ? first : nx;
+}
+template <int QS>
+CNG_DEV unsigned fq_prev_bits(unsigned f, int lane) {
+  const unsigned pv = __shfl_up_sync(FULL, f, 1), last = __shfl_sync(FULL, f, 31) << 1;
+  return (lane == 0 ? last : pv) & ((1u << QS) - 1);
+}
+
+// Sorts a nearly sorted queue and its flags f (odd-even transposition until nothing is out of order).
+template <int QS>
+CNG_DEV void fq_settle(uint64_t (&q)[QS], unsigned& f, int lane) {
   for (int it = 0; it < 32 * QS; ++it) {
     bool bad = false;
 #pragma unroll
     for (int s = 0; s < QS; ++s) bad |= q[s] > fq_next<QS>(q, s, lane);
     if (!__any_sync(FULL, bad)) break;
+    const unsigned fo = __shfl_xor_sync(FULL, f, 1);
+    unsigned take = 0;
 #pragma unroll
     for (int s = 0; s < QS; ++s) {
       const uint64_t o = __shfl_xor_sync(FULL, q[s], 1);
-      q[s] = (lane & 1) ? (o > q[s] ? o : q[s]) : (o < q[s] ? o : q[s]);
+      if ((lane & 1) ? o > q[s] : o < q[s]) {
+        q[s] = o;
+        take |= 1u << s;
+      }
     }
+    f = (f & ~take) | (fo & take);
+    const unsigned fn = fq_next_bits<QS>(f, lane), fp = fq_prev_bits<QS>(f, lane);
+    take = 0;
     uint64_t t[QS];
 #pragma unroll
     for (int s = 0; s < QS; ++s) {
       const uint64_t nx = fq_next<QS>(q, s, lane), pv = fq_prev<QS>(q, s, lane);
-      t[s] = (lane & 1) ? (nx < q[s] ? nx : q[s]) : (pv > q[s] ? pv : q[s]);
+      t[s] = q[s];
+      if ((lane & 1) ? nx < q[s] : pv > q[s]) {
+        t[s] = (lane & 1) ? nx : pv;
+        take |= 1u << s;
+      }
     }
 #pragma unroll
     for (int s = 0; s < QS; ++s) q[s] = t[s];
+    f = (f & ~take) | (((lane & 1) ? fn : fp) & take);
   }
 }
 
-// A key (the same in every lane) with the FP32 rounding of its canonical squared distance.
-template <typename T>
-__device__ __noinline__ uint64_t fk_decide(uint64_t k, const float* qv, const T* X, int dpad, int d, int lane) {
-  if (k & 2) return k;
-  const T* x = X + (int64_t)fk_id(k) * dpad;
-  double c = warp_sqdist_dd(qv, x, d, lane);
-  if (isnan(c)) c = canon_sqdist(qv, x, d);
-  return fk_make(__double2float_rn(c), fk_id(k)) | (k & 1) | 2;
+// Canonical FP64 squared distances of the entries whose bit of `need` is set (bit s: this lane's k[s],
+// s < N), 32 at a time, one per lane.  Returns how many times that was.
+template <typename T, int N>
+__device__ __noinline__ int fk_canon(const uint64_t* k, unsigned need, double* val, const float* qv, const T* X,
+                                      int dpad, int d) {
+  const int lane = threadIdx.x & 31;
+  int total = 0;
+  for (int s = 0; s < N; ++s) total += __popc(__ballot_sync(FULL, need >> s & 1));
+  for (int b = 0; b < total; b += 32) {
+    int32_t id = -1;
+    int o = b;  // rank of slot s's first entry, seen from the batch
+    for (int s = 0; s < N; ++s) {
+      const unsigned m = __ballot_sync(FULL, need >> s & 1);
+      const int r = lane + o;
+      const bool mine = r >= 0 && r < __popc(m);
+      const uint64_t e = __shfl_sync(FULL, k[s], mine ? (int)__fns(m, 0, r + 1) : 0);
+      if (mine) id = fk_id(e);
+      o -= __popc(m);
+    }
+    const double v = id >= 0 ? canon_sqdist(qv, X + (int64_t)id * dpad, d) : 0.0;
+    __syncwarp();
+    o = -b;
+    for (int s = 0; s < N; ++s) {
+      const unsigned m = __ballot_sync(FULL, need >> s & 1);
+      const int r = o + __popc(m & ((1u << lane) - 1));
+      const double t = __shfl_sync(FULL, v, r & 31);
+      if ((need >> s & 1) && r >= 0 && r < 32) val[s] = t;
+      o += __popc(m);
+    }
+  }
+  return (total + 31) / 32;
 }
+
+// The same to within DD_EPS, entry by entry by the whole warp (FP64 only where warp_sqdist_dd gives
+// none and the point is not the query itself; returns fk_canon's count).
+template <typename T, int N>
+__device__ __noinline__ int fk_values(const uint64_t* k, unsigned need, double* val, const float* qv, const T* X,
+                                       int dpad, int d) {
+  const int lane = threadIdx.x & 31;
+  unsigned none = 0;
+  for (int s = 0; s < N; ++s) {
+    unsigned m = __ballot_sync(FULL, need >> s & 1);
+    while (m) {
+      const int l = __ffs(m) - 1;
+      m &= m - 1;
+      const T* x = X + (int64_t)fk_id(__shfl_sync(FULL, k[s], l)) * dpad;
+      double v = warp_sqdist_dd(qv, x, d, lane);
+      if (isnan(v) && warp_rows_equal(qv, x, d, lane)) v = 0.0;
+      if (lane == l) val[s] = v;
+    }
+    if ((need >> s & 1) && isnan(val[s])) none |= 1u << s;
+  }
+  return __any_sync(FULL, none != 0) ? fk_canon<T, N>(k, none, val, qv, X, dpad, d) : 0;
+}
+
+// An entry with the FP32 rounding of its squared distance as key.
+CNG_DEV uint64_t fk_decided(uint64_t k, double v) { return fk_make(__double2float_rn(v), fk_id(k)) | (k & 1) | 2; }
 // Neighbours a <= b, both decided, whose roundings do not settle their order.
 CNG_DEV bool fk_close(uint64_t a, uint64_t b) {
   return a != KINF && b != KINF && (a & b & 2) && (uint32_t)(b >> 33) - (uint32_t)(a >> 33) <= (uint32_t)CLOSE_STEPS;
@@ -169,135 +249,205 @@ CNG_DEV bool fq_has_near(const uint64_t (&q)[QS], uint64_t drop, float band, int
   return __any_sync(FULL, any);
 }
 
-// True if point a comes before b in the order (D, id) of the canonical distance (the arguments are
-// the same in every lane).  FP64 only where the two lie within DD_EPS: one lane's FP64 sum at d = 96
-// takes ~40 us.
-template <typename T>
-__device__ __noinline__ bool canon_before(uint64_t a, uint64_t b, const float* qv, const T* X, int dpad,
-                                          int d, int lane) {
-  const T* xa = X + (int64_t)fk_id(a) * dpad;
-  const T* xb = X + (int64_t)fk_id(b) * dpad;
-  double da = warp_sqdist_dd(qv, xa, d, lane), db = warp_sqdist_dd(qv, xb, d, lane);
-  if (dd_open(da, db)) {
-    da = canon_dist(qv, xa, d);
-    db = canon_dist(qv, xb, d);
+// What fq_fix works on: the queue's keys of a lane and its dropped key; of a query the FP64 sums taken
+// (by up to 32 lanes at once) and whether a key moved; of the warp's queries the entries decided.  In
+// local memory: the search itself is short of registers.
+template <int QS>
+struct FixState {
+  uint64_t q[QS + 1];
+  int sums, moved;
+  unsigned long long decided;
+};
+
+// Which of the pairs `pair` (bit s: the entry k[s] of this lane and the queue's next one, bit QS: the
+// queue's last entry and this lane's dropped key k[QS]) are not in the FP64 order (D, id); FAR is set
+// where the first one's key may not move further.  *sums counts the FP64 sums.
+constexpr unsigned FAR = 1u << 31;
+template <typename T, int QS>
+__device__ __noinline__ unsigned fq_wrong(const uint64_t* k, unsigned pair, int* sums, const float* qv, const T* X,
+                                          int dpad, int d) {
+  constexpr int N = QS + 1;
+  constexpr unsigned QBITS = (1u << QS) - 1, DBIT = 1u << QS, LAST = 1u << (QS - 1);
+  const int lane = threadIdx.x & 31;
+  double val[N], cv[N];
+  for (int s = 0; s < N; ++s) val[s] = cv[s] = 0.0;
+  // the entry (or its value) after slot s of this lane; slot QS: the dropped one, after the queue's last
+  auto first_of = [&](const auto* v, int s) {
+    const auto l = __shfl_sync(FULL, v[QS - 1], 31);
+    return s < QS ? v[s] : l;
+  };
+  auto second_of = [&](const auto* v, int s) {
+    const auto nx = __shfl_down_sync(FULL, v[s], 1);
+    const auto f = __shfl_sync(FULL, v[s + 1 < QS ? s + 1 : s], 0);
+    return s == QS ? v[QS] : (lane == 31 ? f : nx);
+  };
+  auto members = [&](unsigned p) {
+    unsigned need = p | fq_prev_bits<QS>(p & QBITS, lane);
+    if (__any_sync(FULL, p & DBIT) && lane == 31) need |= LAST;
+    return need;
+  };
+  *sums += fk_values<T, N>(k, members(pair), val, qv, X, dpad, d);
+  // pairs that those values leave open: the same row twice, or the canonical distances
+  unsigned open = 0, same = 0;
+  for (int s = 0; s < N; ++s) {
+    const uint64_t ka = first_of(k, s), kb = second_of(k, s);
+    const double va = first_of(val, s), vb = second_of(val, s);
+    const bool op = (pair >> s & 1) && dd_open(va, vb);
+    if (op) open |= 1u << s;
+    unsigned m = __ballot_sync(FULL, op && va == vb);
+    while (m) {
+      const int l = __ffs(m) - 1;
+      m &= m - 1;
+      const int32_t ia = fk_id(__shfl_sync(FULL, ka, l)), ib = fk_id(__shfl_sync(FULL, kb, l));
+      if (warp_rows_equal(X + (int64_t)ia * dpad, X + (int64_t)ib * dpad, d, lane) && lane == l) same |= 1u << s;
+    }
   }
-  return da < db || (da == db && fk_id(a) < fk_id(b));
+  const unsigned canon = open & ~same;
+  if (__any_sync(FULL, canon != 0)) {
+    const unsigned need = members(canon);
+    *sums += fk_canon<T, N>(k, need, cv, qv, X, dpad, d);
+    for (int s = 0; s < N; ++s)
+      if (need >> s & 1) cv[s] = __dsqrt_rn(cv[s]);
+  }
+  unsigned wrong = 0;
+  for (int s = 0; s < N; ++s) {
+    const uint64_t ka = first_of(k, s), kb = second_of(k, s);
+    const double va = first_of(val, s), vb = second_of(val, s);
+    const double ca = first_of(cv, s), cb = second_of(cv, s);
+    if (pair >> s & 1) {
+      const bool idless = fk_id(kb) < fk_id(ka);
+      const bool w = (same >> s & 1)    ? idless
+                     : (canon >> s & 1) ? cb < ca || (cb == ca && idless)
+                                        : vb < va;
+      if (w) wrong |= 1u << s;
+      if (w && s < QS && (uint32_t)(ka >> 33) + 1 - __float_as_uint(__double2float_rn(va)) > (uint32_t)CLOSE_STEPS)
+        wrong |= FAR;
+    }
+  }
+  return wrong;
 }
 
-// Settles the near-ties of the queue qm and of its end against all dropped keys (one per lane); dec
-// counts the entries decided, moves the key moves of the query.  Returns false if the query has to
-// be left to the general kernel.  A call of its own, with the queue through (local) memory: it is
-// rare, and inlined it left the warp in pieces for the rest of the query (20 of 32 lanes to an
+// Settles the near-ties of the queue and of its end against all dropped keys.  Returns false if the
+// query has to be left to the general kernel.  A call of its own, with the queue through local memory:
+// it is rare, and inlined it left the warp in pieces for the rest of the query (20 of 32 lanes to an
 // instruction and twice the instructions on average; 1M x 96, L = 24: 2.1 against 1.0 ms).
+// Only pairs with an entry decided or moved in this call are compared: the others' order was settled
+// when they were.
 template <typename T, int QS>
-__device__ __noinline__ bool fq_fix(uint64_t* qm, uint64_t drop, const float* qv, const T* X, int dpad,
-                                    int d, float band, int* dec_out, int* moves_io) {
+__device__ __noinline__ bool fq_fix(FixState<QS>* fs, const float* qv, const T* X, int dpad, int d, float band,
+                                    int hops) {
+  constexpr int N = QS + 1;  // the queue's entries of a lane and its dropped one
+  constexpr unsigned QBITS = (1u << QS) - 1, DBIT = 1u << QS, LAST = 1u << (QS - 1);
   constexpr uint64_t STEP = 1ull << 33;
   const int lane = threadIdx.x & 31;
-  uint64_t q[QS];
-#pragma unroll
-  for (int s = 0; s < QS; ++s) q[s] = qm[s];
-  int dec = 0, moves = *moves_io;
+  uint64_t q[QS], drop = fs->q[QS];
+  unsigned fresh = 0;  // entries decided, moved or brought in by this call
   bool settled = false;
+#pragma unroll
+  for (int s = 0; s < QS; ++s) q[s] = fs->q[s];
+  auto store = [&]() {
+#pragma unroll
+    for (int s = 0; s < QS; ++s) fs->q[s] = q[s];
+    fs->q[QS] = drop;
+  };
   for (int it = 0; it < FIX_ROUNDS; ++it) {
-    // neighbours within the band: both get their canonical distance
-    bool mark[QS], any = false;
+    // neighbours within the band, both to be decided; within CLOSE_STEPS, to be compared
+    unsigned near = 0, pair = 0, undec = drop & 2 ? 0u : DBIT;
+    const unsigned nfresh = fresh | fq_next_bits<QS>(fresh, lane);
 #pragma unroll
     for (int s = 0; s < QS; ++s) {
-      const uint64_t nx = fq_next<QS>(q, s, lane), pv = fq_prev<QS>(q, s, lane);
-      const bool first = s == 0 && lane == 0;
-      mark[s] = q[s] != KINF && (fk_near(q[s], nx, band) || (!first && fk_near(pv, q[s], band)));
-      any |= mark[s];
+      const uint64_t nx = fq_next<QS>(q, s, lane);
+      if (q[s] != KINF && fk_near(q[s], nx, band)) near |= 1u << s;
+      if ((nfresh >> s & 1) && fk_close(q[s], nx)) pair |= 1u << s;
+      if (!(q[s] & 2)) undec |= 1u << s;
     }
+    near |= fq_prev_bits<QS>(near, lane);
     // the last kept key against every dropped one: while undecided, any of those within the band may
     // come before it
     const uint64_t last = __shfl_sync(FULL, q[QS - 1], 31);
-    const bool dnear = last != KINF && drop != KINF && (drop < last || fk_near(last, drop, band));
-    const bool edge = __any_sync(FULL, dnear);
-    if (edge && lane == 31) mark[QS - 1] = true;
-    if (__any_sync(FULL, any || edge)) {
+    if (last != KINF && drop != KINF && (drop < last || fk_near(last, drop, band))) near |= DBIT;
+    if (fk_close(last, drop)) pair |= DBIT;
+    if (__any_sync(FULL, near & DBIT) && lane == 31) near |= LAST;
+    if (__any_sync(FULL, near != 0)) {
+      const unsigned need = near & undec;
+      fs->decided += __reduce_add_sync(FULL, (unsigned)__popc(need & QBITS));
+      double val[N];
+      store();
+      fs->sums += fk_values<T, N>(fs->q, need, val, qv, X, dpad, d);
 #pragma unroll
-      for (int s = 0; s < QS; ++s) {
-        unsigned mb = __ballot_sync(FULL, mark[s] && !(q[s] & 2));
-        dec += __popc(mb);
-        while (mb) {
-          const int l = __ffs(mb) - 1;
-          mb &= mb - 1;
-          const uint64_t k = fk_decide(__shfl_sync(FULL, q[s], l), qv, X, dpad, d, lane);
-          if (lane == l) q[s] = k;
-        }
-      }
-      unsigned db = __ballot_sync(FULL, dnear && !(drop & 2));
-      while (db) {
-        const int l = __ffs(db) - 1;
-        db &= db - 1;
-        const uint64_t k = fk_decide(__shfl_sync(FULL, drop, l), qv, X, dpad, d, lane);
-        if (lane == l) drop = k;
-      }
-      fq_settle<QS>(q, lane);
+      for (int s = 0; s < QS; ++s)
+        if (need >> s & 1) q[s] = fk_decided(q[s], val[s]);
+      if (need & DBIT) drop = fk_decided(drop, val[QS]);
+      fresh |= need & QBITS;
+      fq_settle<QS>(q, fresh, lane);
       // dropped keys that came out below the last kept one change places with it: each enters at most
       // once, as the last key only falls
       for (;;) {
         const uint64_t lk = __shfl_sync(FULL, q[QS - 1], 31);
-        uint64_t dmin = drop;
+        if (lk == KINF || !__any_sync(FULL, drop < lk)) break;
+        uint64_t in = drop;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
-          const uint64_t y = __shfl_xor_sync(FULL, dmin, o);
-          dmin = y < dmin ? y : dmin;
+          const uint64_t y = __shfl_xor_sync(FULL, in, o);
+          in = y < in ? y : in;
         }
-        if (lk == KINF || dmin >= lk) break;
-        if (lane == __ffs(__ballot_sync(FULL, drop == dmin)) - 1) drop = lk;
-        if (lane == 31) q[QS - 1] = dmin;
-        fq_settle<QS>(q, lane);
+        if (drop == in) drop = lk;
+        if (lane == 31) {
+          q[QS - 1] = in;
+          fresh |= LAST;
+        }
+        fq_settle<QS>(q, fresh, lane);
       }
       continue;
     }
-    // decided neighbours within CLOSE_STEPS: their keys have to be in the FP64 order
-    bool wrong = false, lost = false;
-    int moved = 0;
-#pragma unroll
-    for (int s = 0; s < QS; ++s) {
-      const uint64_t nx = fq_next<QS>(q, s, lane);
-      unsigned cb = __ballot_sync(FULL, fk_close(q[s], nx));
-      while (cb) {
-        const int l = __ffs(cb) - 1;
-        cb &= cb - 1;
-        const uint64_t ka = __shfl_sync(FULL, q[s], l), kb = __shfl_sync(FULL, nx, l);
-        if (canon_before(ka, kb, qv, X, dpad, d, lane)) continue;
-        lost |= (ka >> 33) != (kb >> 33);
-        ++moved;
-        if (lane == l) q[s] += STEP;
-      }
-    }
-    wrong = moved != 0;
-    if (!wrong) {
-      unsigned cb = __ballot_sync(FULL, fk_close(last, drop));
-      while (cb) {
-        const int l = __ffs(cb) - 1;
-        cb &= cb - 1;
-        const uint64_t kd = __shfl_sync(FULL, drop, l);
-        if (canon_before(last, kd, qv, X, dpad, d, lane)) continue;
-        // the dropped point belongs in the queue, the last one out of it for good
-        wrong = true;
-        if (lane == 31) q[QS - 1] = kd;
-        if (lane == l) drop = KINF;
-        break;
-      }
-    }
-    moves += moved;
-    if (lost || moves > CLOSE_STEPS) break;
-    if (!wrong) {
+    if (!__any_sync(FULL, pair != 0)) {
       settled = true;
       break;
     }
-    fq_settle<QS>(q, lane);
-  }
+    store();
+    const int sums = fs->sums;
+    const unsigned wrong = fq_wrong<T, QS>(fs->q, pair, &fs->sums, qv, X, dpad, d);
+    if (__any_sync(FULL, wrong & FAR)) break;
+    if (__any_sync(FULL, wrong & QBITS)) {
 #pragma unroll
-  for (int s = 0; s < QS; ++s) qm[s] = q[s];
-  *dec_out = dec;
-  *moves_io = moves;
-  return settled;
+      for (int s = 0; s < QS; ++s)
+        if (wrong >> s & 1) q[s] += STEP;
+      fresh |= wrong & QBITS;
+      fs->moved = 1;
+      if (fs->sums != sums) fs->sums += MOVE_SUMS;
+    } else if (__any_sync(FULL, wrong & DBIT)) {
+      // a dropped point belongs in the queue, the last one out of it for good
+      uint64_t in = wrong & DBIT ? drop : KINF;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const uint64_t y = __shfl_xor_sync(FULL, in, o);
+        in = y < in ? y : in;
+      }
+      if (drop == in) drop = KINF;
+      if (lane == 31) {
+        q[QS - 1] = in;
+        fresh |= LAST;
+      }
+    } else {
+      settled = true;
+      break;
+    }
+    fq_settle<QS>(q, fresh, lane);
+  }
+  store();
+  return settled && fs->sums <= FP64_SUMS + (QS <= 2 ? hops + hops / 2 : hops / 2);
+}
+
+// The first `cnt` entries' keys without their moves.
+template <typename T, int QS>
+__device__ __noinline__ void fq_round(FixState<QS>* fs, int cnt, const float* qv, const T* X, int dpad, int d) {
+  double val[QS + 1];
+  unsigned need = 0;
+  for (int s = 0; s < QS; ++s)
+    if (s * 32 + (int)(threadIdx.x & 31) < cnt && (fs->q[s] & 2)) need |= 1u << s;
+  fk_values<T, QS + 1>(fs->q, need, val, qv, X, dpad, d);
+  for (int s = 0; s < QS; ++s)
+    if (need >> s & 1) fs->q[s] = fk_decided(fs->q[s], val[s]);
 }
 
 // FP32 squared distances of the query to up to 32 rows (row b named by lane b's v, present when
@@ -371,7 +521,9 @@ __global__ void __launch_bounds__(256, 2) search_float_kernel(SearchArgs a) {
   }
   const int hmask = a.hash_slots - 1, L = a.L, dpad = a.dpad;
   const T* X = reinterpret_cast<const T*>(a.X);
-  unsigned long long t_ndc = 0, t_hops = 0, t_f64 = 0, t_stop = 0;
+  unsigned long long t_ndc = 0, t_hops = 0, t_stop = 0;
+  FixState<QS> fs;
+  fs.decided = 0;
 
   // each warp takes query (its index) first, then queries nw + (queue head) as it finishes them
   const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
@@ -411,7 +563,7 @@ __global__ void __launch_bounds__(256, 2) search_float_kernel(SearchArgs a) {
     int32_t pf_u = -1;  // predicted next hop vertex and its out-list
     int32_t pf[SQ_ROWSLOTS];
     bool left = false;  // to the general kernel
-    int moves = 0;
+    fs.sums = fs.moved = 0;
     for (;;) {
       __syncwarp();
       const int idx = fq_first_open<QS>(q);
@@ -504,16 +656,13 @@ __global__ void __launch_bounds__(256, 2) search_float_kernel(SearchArgs a) {
         const int32_t old_kth = LEARN && old_len >= a.k ? fk_id(fq_get<QS>(q, a.k - 1)) : -1;
         const uint64_t drop = fq_merge<QS>(q, __shfl_sync(FULL, kb, 31 - lane), lane);
         if (!qexact && fq_has_near<QS>(q, drop, a.band, lane)) {
-          uint64_t qm[QS];
-          int dec, mv = moves;
 #pragma unroll
-          for (int s = 0; s < QS; ++s) qm[s] = q[s];
-          left = !fq_fix<T, QS>(qm, drop, qv, X, dpad, a.d, a.band, &dec, &mv);
+          for (int s = 0; s < QS; ++s) fs.q[s] = q[s];
+          fs.q[QS] = drop;
+          left = !fq_fix<T, QS>(&fs, qv, X, dpad, a.d, a.band, hops);
 #pragma unroll
-          for (int s = 0; s < QS; ++s) q[s] = qm[s];
-          moves = mv;
+          for (int s = 0; s < QS; ++s) q[s] = fs.q[s];
           flags |= 1;
-          t_f64 += dec;
           __syncwarp();
           if (left) break;
         }
@@ -585,7 +734,14 @@ __global__ void __launch_bounds__(256, 2) search_float_kernel(SearchArgs a) {
       __syncwarp();
       continue;
     }
-    // results
+    // results; keys that moved give way to their roundings
+    if (__any_sync(FULL, fs.moved)) {
+#pragma unroll
+      for (int s = 0; s < QS; ++s) fs.q[s] = q[s];
+      fq_round<T, QS>(&fs, min(a.k, len), qv, X, dpad, a.d);
+#pragma unroll
+      for (int s = 0; s < QS; ++s) q[s] = fs.q[s];
+    }
 #pragma unroll
     for (int s = 0; s < QS; ++s) {
       const int t = s * 32 + lane;
@@ -608,7 +764,7 @@ __global__ void __launch_bounds__(256, 2) search_float_kernel(SearchArgs a) {
   if (lane == 0) {
     atomicAdd(&a.tot[0], t_ndc);
     atomicAdd(&a.tot[1], t_hops);
-    if (t_f64) atomicAdd(&a.tot[2], t_f64);
+    if (fs.decided) atomicAdd(&a.tot[2], fs.decided);
     if (t_stop) atomicAdd(&a.tot[3], t_stop);
   }
 }

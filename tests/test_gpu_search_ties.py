@@ -29,3 +29,22 @@ def test_points_of_few_levels(levels, d, L, dtype):
     assert st["exact_int"] == 0
     _search_check(X, Q, idx, cng, min(10, L), L)
     cng.cng_free(idx)
+
+
+def test_copies_cost_no_fp64_sums():
+    """Every point stored twice: the pairs' order is their ids', found without FP64 sums.  Searches
+    take at most 20 times those of single points (2 measured; with every tied pair of the queue
+    compared in FP64 after each hop it was 330 times)."""
+    need_gpu()
+    cng = lib()
+    rng = np.random.default_rng(103)
+    X = rng.standard_normal((8000, 96)).astype(np.float32)
+    Q = tensor(rng.standard_normal((1000, 96)).astype(np.float32))
+    ms = []
+    for rows in (X, np.tile(X[:4000], (2, 1))):
+        idx, _ = cng.cng_build(tensor(rows), alpha=1.2, R=24, L=64, repair_slots=32, connect_L=64)
+        runs = [cng.cng_search(idx, Q, k=10, L=128, warps_per_block=4, with_stats=True)["stats"]["ms"]
+                for _ in range(4)]
+        ms.append(min(runs))
+        cng.cng_free(idx)
+    assert ms[1] <= 20 * ms[0], ms
