@@ -533,11 +533,12 @@ bool search_plan(SearchArgs& a, int wpb, int hash_slots, SearchPlan* p) {
   a.warp_smem = search_warp_smem(a.dpad, a.L, hash_slots);
   a.warp_smem_fast = 0;
   // a register-queue kernel: L <= 256 and row stride <= 96; the 8-bit one for exact data with
-  // 8-bit rows.  It needs the list of deferred queries.
+  // 8-bit rows.  It needs the list of deferred queries, unless the queries are stored points of
+  // such data (none is deferred).
   int qs = 0;
-  if (a.defer && a.R <= SQ_ROWSLOTS * 32 && a.k <= a.L)
-    qs = a.L <= 32 ? 1 : a.L <= 64 ? 2 : a.L <= 128 ? 4 : a.L <= 256 ? 8 : 0;
   const bool u8 = a.U && a.exact && a.dtype == CNG_F32;
+  if ((a.defer || (u8 && a.qids)) && a.R <= SQ_ROWSLOTS * 32 && a.k <= a.L)
+    qs = a.L <= 32 ? 1 : a.L <= 64 ? 2 : a.L <= 128 ? 4 : a.L <= 256 ? 8 : 0;
   if (qs) {
     const bool learn = a.model || a.trace_feats;
     a.warp_smem_fast = u8 ? search_fast_warp_smem(a.u8w, hash_slots) : search_float_warp_smem(a.dpad, hash_slots);
