@@ -746,7 +746,9 @@ static void schedule(const TcScreenArgs& a, int bn, int ntiles, ResParams* p) {
     // a part worth a cut: some tiles of its own, and a rank well below Lp
     const int prev = p->npart ? p->part_end[p->npart - 1] : 0;
     if (t - prev < 4 || t >= ntiles) continue;
-    const int rank = sample_rank(a.Lp, (double)t * bn / (double)a.n);
+    // by the part's sampling rate: the columns cut off at its last whole tile are those of one region
+    // of the order, so rows far from it see all of their sample
+    const int rank = sample_rank(a.Lp, (double)end / (double)a.n);
     if (rank * 4 > a.Lp * 3) continue;
     p->part_end[p->npart] = t;
     p->part_rank[p->npart++] = rank;
