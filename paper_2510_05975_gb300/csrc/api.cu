@@ -463,6 +463,10 @@ static float bits_to_float(uint32_t b) {
   return f;
 }
 
+// Rows from which the screen's scratch and operands are freed as soon as they are not needed (a free
+// waits for the GPU: with 10,000 rows a build took 5.6 ms, against 5.4 with all of it freed at the end).
+constexpr int64_t FREE_EARLY = 1 << 17;
+
 // The columns' tile image in a sampled order of perm (device ids; *order: position -> id, *pos: its
 // inverse if wanted) and the parts' sizes, for screens whose rows fit the resident kernel.
 // Synchronises.
@@ -470,12 +474,14 @@ static cng_status sampled_image(DevPool& pool, const ResShape& r, int fp16, cons
                                 int64_t n, int kpad, const int32_t* perm, void** image,
                                 const int32_t** order, const int32_t** pos, int64_t* part_count,
                                 cudaStream_t s) {
+  DevPool local;
+  DevPool& tmp = n >= FREE_EARLY ? local : pool;
   int32_t *out, *inv = nullptr, *cnt;
   char *scr, *img;
   CK(pool.alloc(&out, (size_t)n));
   if (pos) CK(pool.alloc(&inv, (size_t)n));
-  CK(pool.alloc(&cnt, 4));
-  CK(pool.alloc(&scr, sample_scratch_bytes(n)));
+  CK(tmp.alloc(&cnt, 4));
+  CK(tmp.alloc(&scr, sample_scratch_bytes(n)));
   CK(launch_sample_order(perm, n, out, inv, cnt, scr, s));
   CK(pool.alloc(&img, res_image_bytes(r, n)));
   CK(launch_tile_image(r, fp16 != 0, pr.tc, kpad, pr.nb, out, n, img, s));
@@ -505,9 +511,12 @@ static cng_status apply_order(DevPool& pool, Prepared* pr, int dtype, int64_t n,
     char* rimg;
     CK(pool.alloc(&perm, (size_t)n));
     if (kd) {
+      DevPool local;
+      DevPool& tmp = n >= FREE_EARLY ? local : pool;
       char* oscr;
-      CK(pool.alloc(&oscr, order_scratch_bytes(n)));
+      CK(tmp.alloc(&oscr, order_scratch_bytes(n)));
       CK(launch_order(pr->xs, dtype, n, d, dpad, perm, oscr, s));
+      if (n >= FREE_EARLY) CK(cudaStreamSynchronize(s));
     } else {
       CK(launch_iota(perm, n, s));
     }
@@ -793,6 +802,10 @@ extern "C" cng_status cng_build(const void* points, int32_t dtype, int64_t n, in
     if (st != CNG_OK) return st;
   }
   // screening operands are no longer needed
+  if (ki.res.kt > 0 && n >= FREE_EARLY) {  // the columns' image
+    cudaFree(const_cast<void*>(ki.tc_cols));
+    pool.release(const_cast<void*>(ki.tc_cols));
+  }
   if (pr.tc) { cudaFree(pr.tc); pool.release(pr.tc); pr.tc = nullptr; }
   if (beam) {
     // Alg. 3 phase 2 (Sec. 4.1): beam search for every point on G0 from the navigating node;
@@ -1664,6 +1677,10 @@ extern "C" cng_status cng_knn(const float* base, int64_t n, const float* rows, i
     st = sampled_image(pool, ki.res, ki.tc_fp16, pb, n, kpad, input, &cimg, &ki.col_perm, nullptr,
                        ki.part_count, s);
     if (st != CNG_OK) return st;
+    if (n >= FREE_EARLY) {  // the image replaces the copy (sampled_image has waited for its reads)
+      cudaFree(pb.tc);
+      pool.release(pb.tc);
+    }
     CK(pool.alloc(&rimg, res_image_bytes(ki.res, m)));
     CK(launch_tile_image(ki.res, ki.tc_fp16 != 0, prw.tc, kpad, prw.nb, nullptr, m, rimg, s));
     ki.tc_rows = rimg;
