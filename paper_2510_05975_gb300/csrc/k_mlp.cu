@@ -31,6 +31,7 @@ constexpr int MA = 32;   // samples per CTA of the forward / backward kernel
 constexpr int MF = 256;  // its threads
 constexpr int MO = 64 / (MF / 32);  // outputs of a layer per warp
 constexpr int MG = 8;    // CTAs per group of the gradient kernel
+constexpr int MC = 1024; // groups whose activations are held at once (144 MB)
 
 CNG_DEV uint64_t splitmix64(uint64_t x) {
   x += 0x9E3779B97F4A7C15ull;
@@ -156,7 +157,7 @@ __global__ void standardise_kernel(float* __restrict__ X, int64_t N, const float
 }
 
 // ---- forward + backward --------------------------------------------------------------------------
-// Activations and gradients of a batch, [samples rounded up to MT][..]: x 16, h1, h2, g1 (dL/da1) and
+// Activations and gradients of up to MC groups, [samples rounded up to MT][..]: x 16, h1, h2, g1 (dL/da1) and
 // g2 (dL/da2) 64 each, dz and the loss 1 each.
 struct MlpActs {
   float *x, *h1, *h2, *g1, *g2, *dz, *ls;
@@ -164,8 +165,8 @@ struct MlpActs {
 CNG_DEV void put4(float* p, const float* v) {
   *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
 }
-static MlpActs acts_of(float* p, int B) {
-  const size_t n = (size_t)mlp_parts(B) * MT;
+static MlpActs acts_of(float* p, int groups) {
+  const size_t n = (size_t)groups * MT;
   MlpActs a;
   a.x = p;
   a.h1 = a.x + n * 16;
@@ -177,23 +178,23 @@ static MlpActs acts_of(float* p, int B) {
   return a;
 }
 
-// Rows drawn by hash of (seed, step, slot), or 0..B-1 (seed 0).  Lane = sample; warp w computes
+// Samples s0 .. of the batch: rows drawn by hash of (seed, step, slot), or 0..B-1 (seed 0).  Lane = sample; warp w computes
 // outputs MO w .. + MO - 1 of each layer and keeps them in registers for the backward pass.
 __global__ void __launch_bounds__(MF)
 mlp_fwd_bwd_kernel(const float* __restrict__ P, const float* __restrict__ X, const float* __restrict__ Y,
-                   int64_t N, int B, uint64_t seed, int64_t step, float inv_scale, MlpActs A) {
+                   int64_t N, int B, int s0, uint64_t seed, int64_t step, float inv_scale, MlpActs A) {
   __shared__ __align__(16) float w[MLP_NPARAMS_PAD];
   __shared__ float h1[MA * 65];  // [sample][65] (pad: conflict-free columns)
   __shared__ float h2[MA * 65];  // later dL/da2
   __shared__ float dzs[MA];
   const int t = threadIdx.x, lane = t & 31, o0 = (t >> 5) * MO;
-  const int64_t s = (int64_t)blockIdx.x * MA + lane;
-  const bool live = s < B;
+  const int s = (int)blockIdx.x * MA + lane, slot = s0 + s;
+  const bool live = slot < B;
   int64_t row = 0;
   if (live) {
-    row = seed ? (int64_t)(splitmix64(seed ^ ((uint64_t)step * 0x100000001B3ull + (uint64_t)s)) %
+    row = seed ? (int64_t)(splitmix64(seed ^ ((uint64_t)step * 0x100000001B3ull + (uint64_t)slot)) %
                            (uint64_t)N)
-               : s;
+               : slot;
   }
   float x[16];
 #pragma unroll
@@ -460,22 +461,26 @@ __global__ void pack_model_kernel(const float* __restrict__ P, const float* __re
 // ---- host-side launchers ---------------------------------------------------------------------------
 int mlp_parts(int B) { return (B + MT - 1) / MT; }
 size_t mlp_scratch_floats(int B) {
-  const size_t n = (size_t)mlp_parts(B) * MT;
+  const size_t n = (size_t)std::min(mlp_parts(B), MC) * MT;
   return (size_t)mlp_parts(B) * (MLP_NPARAMS + 1) + 4 + n * (16 + 4 * 64 + 2);
 }
 
-// scratch: the groups' losses, their partial gradients, the activations (16-byte aligned)
+// scratch: the groups' losses, their partial gradients, the activations of MC groups (16-byte aligned)
 static cudaError_t launch_partials(const float* P, const float* X, const float* Y, int64_t N, int B,
                                    uint64_t seed, int64_t step, float* scratch, float** part,
                                    float** part_loss, cudaStream_t s) {
   const int parts = mlp_parts(B);
   *part_loss = scratch;
   *part = scratch + parts;
-  const MlpActs A = acts_of(scratch + ((size_t)parts * (MLP_NPARAMS + 1) + 3) / 4 * 4, B);
-  count_launch();
-  mlp_fwd_bwd_kernel<<<parts * (MT / MA), MF, 0, s>>>(P, X, Y, N, B, seed, step, 1.f / (float)B, A);
-  count_launch();
-  mlp_group_grad_kernel<<<dim3(parts, MG), 256, 0, s>>>(A, *part, *part_loss);
+  const MlpActs A = acts_of(scratch + ((size_t)parts * (MLP_NPARAMS + 1) + 3) / 4 * 4, std::min(parts, MC));
+  for (int g0 = 0; g0 < parts; g0 += MC) {
+    const int groups = std::min(parts - g0, MC);
+    count_launch();
+    mlp_fwd_bwd_kernel<<<groups * (MT / MA), MF, 0, s>>>(P, X, Y, N, B, g0 * MT, seed, step,
+                                                         1.f / (float)B, A);
+    count_launch();
+    mlp_group_grad_kernel<<<dim3(groups, MG), 256, 0, s>>>(A, *part + (size_t)g0 * MLP_NPARAMS, *part_loss + g0);
+  }
   return cudaGetLastError();
 }
 
