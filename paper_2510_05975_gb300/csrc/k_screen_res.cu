@@ -765,20 +765,26 @@ static int list_cap(int Lp, int step) {
   return caps[std::min(3, ci + step)] * 32;
 }
 
-// Column split for launches whose row blocks leave SMs idle (fewer than 4 per SM): the split and the sample parts swept whole by each unit that minimise
-//   waves x (unit overhead + sample tiles + other tiles / splits + hits),
-// in tiles of ~850 cycles; a hit per row costs ~6 tiles (32 rows append in turn), a unit's operand
-// load and final lists ~40, merging the splits' lists ~60.  10,000 rows against 1M x 128 (40 row
-// blocks): 3 splits with the 1/16 sample, 8.0 -> 4.2 ms.  With many row blocks nothing is gained: the
-// sample would be swept once per split.
-static void split_columns(int64_t nrb, int bn, int64_t n, int Lp, int cap, ResParams* p) {
+// Column split for launches whose row blocks leave half of the SMs or more idle: the split and the
+// sample parts swept whole by each unit, at most one unit per SM, that minimise
+//   unit overhead + sample tiles + other tiles / splits + hits
+// in tiles of ~850 cycles; a hit per row costs ~6 tiles (the 32 rows of a warp append in turn; fewer
+// rows, less), a unit's operand load and final lists ~40, merging the splits' lists ~60.  A list that
+// starts empty takes its first `cap` columns at once, then a buffer's worth per cut, with the
+// threshold of the last cut.  Screen of m rows, split / whole (ms): 1M x 128, k = 100: m = 1 0.42 / 5.5,
+// 1,000 1.3 / 7.8, 5,000 2.6 / 7.8, 10,000 4.3 / 7.9; k = 10: 1,000 1.2 / 6.8, 10,000 3.8 / 6.9; 100k x 96,
+// k = 100: 1,000 0.49 / 1.95, 10,000 1.2 / 2.0.  More than one unit per SM lost: 20,000 rows in 237 units
+// 8.4 / 7.9 (k = 10: 10.1 / 6.9), 39,000 rows in 306 16.1 / 15.2, so from 77 row blocks on nothing is split.
+static void split_columns(int64_t m, int bn, int64_t n, int Lp, int cap, ResParams* p) {
   p->nsplit = 1;
   p->pre = 0;
-  const int64_t sms = num_sms();
-  if (nrb >= 4 * sms) return;
-  const double hit = 6.0, unit = 40.0, merge = 60.0;
-  auto fill = [&](double cols, int rank) {  // appends of a list that starts empty: rows append at once
-    return 0.4 * (cols <= cap ? cols : cap + rank * std::log(cols / cap));
+  const int64_t sms = num_sms(), nrb = (m + RS_BM - 1) / RS_BM;
+  if (2 * nrb > sms) return;
+  const double hit = std::max(0.5, 6.0 * (double)std::min<int64_t>(m, 32) / 32.0), unit = 40.0, merge = 60.0;
+  auto fill = [&](double cols, int rank) {
+    const double more = cap - bn - rank;  // appends between two cuts
+    return 0.4 * std::min<double>(cols, cap) +
+           (cols > cap ? more * std::log(cols / cap) / std::log1p(more / rank) : 0.0);
   };
   // appends per row up to the end of each part
   double upto[RES_PARTS], frac[RES_PARTS];
@@ -787,15 +793,14 @@ static void split_columns(int64_t nrb, int bn, int64_t n, int Lp, int cap, ResPa
     upto[i] = i == 0 ? fill(frac[0] * (double)n, p->part_rank[0])
                      : upto[i - 1] + p->part_rank[i - 1] * (frac[i] / frac[i - 1] - 1.0);
   }
-  double best = (double)((nrb + sms - 1) / sms) * (unit + p->ntiles + hit * upto[p->npart - 1]);
+  double best = unit + p->ntiles + hit * upto[p->npart - 1];
   int best_k = -2;
   for (int k = -1; k + 1 < p->npart; ++k) {
     const int pre = k < 0 ? 0 : p->part_end[k];
-    for (int64_t sp = 2; sp * nrb <= 4 * sms && sp <= sms && sp * 4 <= p->ntiles - pre; ++sp) {
+    for (int64_t sp = 2; sp * nrb <= sms && sp * 4 <= p->ntiles - pre; ++sp) {
       const double h = k < 0 ? fill((double)n / (double)sp, Lp)
                              : upto[k] + p->part_rank[k] * (1.0 / frac[k] - 1.0) / (double)sp;
-      const double c = merge + (double)((nrb * sp + sms - 1) / sms) *
-                                   (unit + pre + (double)(p->ntiles - pre) / (double)sp + hit * h);
+      const double c = merge + unit + pre + (double)(p->ntiles - pre) / (double)sp + hit * h;
       if (c < best) {
         best = c;
         best_k = k;
@@ -834,7 +839,7 @@ static void plan_res(const TcScreenArgs& a, int cap_step, bool split, ResParams*
   schedule(a, bn, p->ntiles, p);
   p->nsplit = 1;
   p->pre = 0;
-  if (split) split_columns((a.m + RS_BM - 1) / RS_BM, bn, a.n, a.Lp, p->cap, p);
+  if (split) split_columns(a.m, bn, a.n, a.Lp, p->cap, p);
   if (p->nsplit > 1) p->cap = p->cap <= 512 ? 512 : 768;  // the capacities split kernels are built for
 }
 

@@ -35,3 +35,18 @@ def test_beam_candidates_of_byte_rows_use_the_register_queue():
 
         counts.append(_launches(cng, build))
     assert counts[0] == counts[1] + 1
+
+
+def test_column_splits_stop_at_one_unit_per_sm():
+    """k-NN of up to 76 row blocks of 256 splits the columns (one more launch, which merges the splits'
+    lists); from 77 row blocks on a split would give an SM two units in turn, which is slower."""
+    need_gpu()
+    cng = lib()
+    rng = np.random.default_rng(112)
+    X, Q = tensor(rng.standard_normal((1_000_000, 16)).astype(np.float32)), rng.standard_normal((60_000, 16))
+    counts = {}
+    for m in (1, 1000, 10_000, 20_000, 39_000, 60_000):
+        rows = tensor(Q[:m].astype(np.float32))
+        counts[m] = _launches(cng, lambda: cng.cng_knn(X, 10, rows=rows))
+    assert counts[1] == counts[1000] == counts[10_000] == counts[60_000] + 1
+    assert counts[20_000] == counts[39_000] == counts[60_000]
