@@ -336,7 +336,8 @@ static cng_status run_knn(const KnnInputs& in, int32_t* out_ids, float* out_dist
     sm.rb = in.rb_rows;
     sm.rbmax = in.rbmax;
     sm.normmax = in.normmax;
-    // K terms, 2^-23 per add (the norm pieces among them when they are part of the operands)
+    // K terms, 2^-23 per add (the norm pieces among them when they are part of the operands; what the
+    // pieces leave out is counted apart)
     sm.acc_err = (float)(in.res.kt > 0 ? in.res.kt + 16 : in.kpad + 8) * 1.1920929e-7f;
     sm.abs_err = in.res.kt > 0 && in.tc_fp16 ? RES_PIECE_ERR : 0.f;
     sm.scale2 = in.scale2;
@@ -902,7 +903,7 @@ extern "C" cng_status cng_build(const void* points, int32_t dtype, int64_t n, in
   CK(pool.alloc(&adj, (size_t)n * Rs));
   CK(pool.alloc(&deg, (size_t)n));
   int32_t* big_list;
-  CK(pool.alloc(&big_list, 2 * (size_t)n));  // big list + the 8-bit merge's middle list
+  CK(pool.alloc(&big_list, 2 * (size_t)n));  // big list + the middle list of the merges
   CK(launch_reverse(fwd, fdeg, n, R, indeg, off, cursor, inl, bsum, ctr, s));
   MergeScratch ms{};  // merged sets listed for the Gram-tile (8-bit rows) or all-pairs re-prune
   if (!P.adaptive && (gram_prune_ok(u8, u8w, 128, R) || (!u8 && pairs_prune_ok(256, R, false)))) {

@@ -39,7 +39,7 @@ struct Counters {
   uint32_t screen_err_bits;
   int nbig;        // nodes whose merged set exceeds the shared-memory capacity
   int max_indeg;
-  int nmid;        // 8-bit merge: nodes deferred from the 128-entry to the 256-entry pass
+  int nmid;        // merges: nodes left to the next pass (8-bit rows: above 128 entries; float: above 256)
   unsigned long long alpha_steps;  // adaptive pruning: sum over phase-2 points of the alpha step
   int nre;         // merged sets listed for the re-prune (Gram tile of 8-bit rows, all-pairs kernel)
   int nsmall;      // FP16 merge: sets of up to 128 listed for the Gram tile

@@ -8,11 +8,13 @@
 // Operands.  Each operand row has kt = d + 6 elements rounded up to 16: the d coordinates, then
 // six norm pieces.  A column holds p_0..p_5 with sum c_i p_i = ||y_b||^2 / 2 to max(2^-35 of it,
 // 2^-25) in FP16 (operands are scaled so that the largest coordinate exceeds 4096 unless they are
-// integers, and the certification counts the absolute part) and to 2^-48 of it in BF16, a row holds the constants -c_i, so the accumulator is a = <x_b, y_b> - ||y_b||^2 / 2 = -s / 2 and
-// the epilogue only compares it with the row's threshold (an FMA and a shared-memory norm load per
-// score in the epilogue's fast path cost more than the extra 16 K elements of the MMA).  Integer
-// operands with ||x||^2 < 2^23 stay exact: pieces, products and sums are multiples of 1/2 below
-// 2^23.
+// integers, and the certification counts the absolute part) and to 2^-48 of it in BF16, a row holds
+// the constants -c_i, so the accumulator is a = <x_b, y_b> - ||y_b||^2 / 2 = -s / 2 and the epilogue
+// only compares it with the row's threshold (an FMA and a shared-memory norm load per score in the
+// epilogue's fast path cost more than the extra 16 K elements of the MMA).  Integer
+// operands with ||x||^2 < 2^23 and distances D^2 < 2^24 (d span^2 < 2^24, span the range of the
+// coordinates) stay exact: pieces, products and sums are multiples of 1/2, a partial inner product is
+// below 2^23 in magnitude, and the accumulator is (||x||^2 - D^2) / 2, between -2^23 and 2^22.
 //
 // Column order.  Columns are swept in a sampled order: a pseudo-random 1/64 of them first, then up
 // to 1/16, 1/4 and all (each part in locality order).  After a part that holds the fraction f of
@@ -34,7 +36,8 @@
 // A in TMEM: it leaves shared memory's bandwidth and 72 KB of it to the column tiles.  One issuer
 // per accumulator: after its MMAs an issuer spends ~350 cycles in commits and barrier waits in
 // which the tensor pipe, which queues only a few MMAs, would idle (one issuer for all: 1,680
-// cycles per 256 x 80 tile; two: 1,260; four: 840, against 890 for the 18 MMAs alone at 49 each).
+// cycles per 256 x 80 tile; two: 1,260; four: 840, where the 18 MMAs take 720 at the pipe's nominal
+// 8,192 operations a cycle).
 //
 // Bound: without hits the tensor pipe (1,900 TFLOP/s of 2 m n d at d = 128); the appends add ~40%.
 // 1M x 128, L' = 160, self: 202 ms, 1,265 TFLOP/s of 2 n^2 d (0.74 of the measured sustained bf16
