@@ -321,15 +321,18 @@ def hbm_kernels(w, X, st, ndc_sum, hops_sum, search_ms, peak, src):
 # DRAM bytes (read + write) of one full-size screen launch from a one-pass ncu capture, keyed by
 # (workload, digest of the screen kernel's source): a changed kernel has no entry, so its
 # traffic is reported as null until it is captured again.
-SCREEN_DRAM_BYTES = {("sift1m", "2fde0dbd24a93892"): 18.55e9 + 20.29e9}
+SCREEN_DRAM_BYTES = {("sift1m", "b35c09bb4c7d4c48"): 15.33e9 + 12.17e9}
 
 
-def screen_digest() -> str:
+def screen_digest(d: int) -> str:
+    """Digest of the sources of the screen kernel that rows of d coordinates run on."""
     import hashlib
 
-    path = os.path.join(ROOT, "paper_2510_05975_gb300", "csrc", "k_screen_res.cu")
-    with open(path, "rb") as f:
-        return hashlib.sha256(f.read()).hexdigest()[:16]
+    h = hashlib.sha256()
+    for name in ("k_screen_res.cu" if d <= 250 else "k_screen_tc.cu", "screen_common.cuh", "screen_tc.h"):
+        with open(os.path.join(ROOT, "paper_2510_05975_gb300", "csrc", name), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:16]
 
 
 def main():
@@ -647,10 +650,10 @@ def main():
     achieved = flops / t_screen / 1e12
     traffic = None
     if roof["bound"] == "tensor" and screen == cng.CNG_SCREEN_TC:
-        traffic = SCREEN_DRAM_BYTES.get((args.workload, screen_digest()))
+        traffic = SCREEN_DRAM_BYTES.get((args.workload, screen_digest(w.d)))
     roof.update({"kernel": "candidate screen", "achieved": achieved, "frac": achieved / roof["peak"],
                  "traffic": traffic, "traffic_unit": "bytes per launch (ncu dram read + write)",
-                 "kernel_digest": screen_digest(),
+                 "kernel_digest": screen_digest(w.d),
                  "algorithmic": "2*n*n*d flops per launch"})
 
     hbm = hbm_kernels(w, X, last_stats, ndc_sum_f, hops_sum_f, f_ms, pk["hbm_gbs"], src)
