@@ -50,9 +50,10 @@ struct SearchArgs {
   const uint8_t* U;         // [n][4 u8w]
   const uint8_t* QU;        // queries in the same form [nq][4 u8w] (unused with qids)
   int u8w;                  // 8, 16, 24 or 32
-  // two-kernel launch (SearchPlan::fast_qs > 0): the register-queue kernel serves every exact
-  // query and appends the others to defer[] (>= nq entries, counter[1] counts them); the general
-  // kernel then serves the list qlist[0 .. *nq_dev) with counter[2] as its queue head
+  // two-kernel launch (SearchPlan::fast_qs > 0): the register-queue kernel serves what it can (8-bit
+  // rows: every exact query; float rows: queries whose near-ties it settles) and appends the others to
+  // defer[] (>= nq entries, counter[1] counts them; null only for stored points on 8-bit rows); the
+  // general kernel then serves the list qlist[0 .. *nq_dev) with counter[2] as its queue head
   int32_t* defer;
   const int32_t* qlist;
   const int* nq_dev;
